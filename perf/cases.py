@@ -67,7 +67,7 @@ def listed():
     ]
 
 
-MOST_BYTES = 1.4e11  # of one drawn case
+MOST_BYTES = 1.2e11  # of one drawn case
 
 
 def _log(rng, lo, hi):
