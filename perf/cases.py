@@ -107,7 +107,7 @@ def draw(rng):
         elif rng.random() < 0.5:  # half of the grids have the rounded rows of a benchmark
             nx = (nx + 15) // 16 * 16
         sr32 = storage == "f32" and not inplace and nx * ny * nz < 1e5 and rng.random() < 0.2
-        most = MOST_BYTES / (2 * Q * ELEM[storage] * nx * ny * nz)
+        most = MOST_BYTES / ((2 * Q * ELEM[storage] + 28) * nx * ny * nz)
         steps = 2 * int(max(2, min(rng.randrange(4, 101), most / 2)))
     return _case(None, nx, ny, nz, steps, kind=kind, Q=Q, storage=storage, walls=walls, force=force,
                  tau=tau, others=others, inplace=inplace, sr32=sr32)
