@@ -192,12 +192,12 @@ __global__ void __launch_bounds__(128, 3) adjoint2_kernel(const StepIO<T> io, co
 // lam_a = u.e_a - |u|^2 / 2, and the direct term dJ/dF += u / 2
 // (u = (j + F/2) / rho).
 template <int Q, typename T>
-__global__ void __launch_bounds__(128) energy_seed_kernel(const T *__restrict__ buf,
+__global__ void __launch_bounds__(128) energy_seed_kernel(const StepIO<T> io,
                                                           const StepArgs a, AdjointArgs g) {
     int x, y, z;
     if (!cell_coords(a.g, x, y, z)) return;
     float f[Q];
-    gather<Q, T>(buf, a.g, pull_sources(a.g, x, y, z), f);
+    gather<Q, T>(io, a.g, x, y, z, f);
     float drho, jx, jy, jz, Fx, Fy, Fz;
     moments<Q>(f, drho, jx, jy, jz);
     const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
@@ -224,14 +224,14 @@ __global__ void __launch_bounds__(128) energy_seed_kernel(const T *__restrict__ 
 //     lam_a = g_rho + sum_i (e_ai - u_i) g_u_i / rho,
 // and the direct term dJ/dF_i += g_u_i / (2 rho) (u carries F/2).
 template <int Q, typename T>
-__global__ void __launch_bounds__(128) macro_seed_kernel(const T *__restrict__ buf,
+__global__ void __launch_bounds__(128) macro_seed_kernel(const StepIO<T> io,
                                                          const StepArgs a, AdjointArgs g,
                                                          const float *__restrict__ g_rho,
                                                          const float *__restrict__ g_u) {
     int x, y, z;
     if (!cell_coords(a.g, x, y, z)) return;
     float f[Q];
-    gather<Q, T>(buf, a.g, pull_sources(a.g, x, y, z), f);
+    gather<Q, T>(io, a.g, x, y, z, f);
     float drho, jx, jy, jz, Fx, Fy, Fz;
     moments<Q>(f, drho, jx, jy, jz);
     const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
@@ -256,35 +256,24 @@ __global__ void __launch_bounds__(128) macro_seed_kernel(const T *__restrict__ b
 }
 
 // Per-block partial sums of rho |u|^2 / 2 (slot 0 of each 4-double record),
-// rows assigned to blocks as in the conservation reduction.
+// cells assigned to blocks as in the conservation reduction.
 template <int Q, typename T>
-__global__ void __launch_bounds__(kRedThreads) energy_kernel(const T *__restrict__ buf,
-                                                             const StepArgs a,
-                                                             double *__restrict__ part) {
+__global__ void __launch_bounds__(128, 8) energy_kernel(const StepIO<T> io, const StepArgs a,
+                                                        double *__restrict__ part) {
     const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
-    const long long rows = (long long)a.g.ny * a.g.nz;
-    double acc = 0.0;
-    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-        const int y = int(row % a.g.ny), z = int(row / a.g.ny);
-        for (int x = threadIdx.x; x < a.g.nx; x += blockDim.x) {
-            float f[Q];
-            gather<Q, T>(buf, a.g, pull_sources(a.g, x, y, z), f);
-            float drho, jx, jy, jz, Fx, Fy, Fz;
-            moments<Q>(f, drho, jx, jy, jz);
-            cell_force(a, row * a.g.nx + x, N, Fx, Fy, Fz);
-            const float px = jx + 0.5f * Fx, py = jy + 0.5f * Fy, pz = jz + 0.5f * Fz;
-            acc += double(0.5f * (px * px + py * py + pz * pz) / (1.0f + drho));
-        }
-    }
-    __shared__ double sh[kRedThreads];
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        part[4 * blockIdx.x] = sh[0];
+    double acc[1] = {0.0};
+    for_cells(a.g, [&](int x, int y, int z, long long c) {
+        float f[Q];
+        gather<Q, T>(io, a.g, x, y, z, f);
+        float drho, jx, jy, jz, Fx, Fy, Fz;
+        moments<Q>(f, drho, jx, jy, jz);
+        cell_force(a, c, N, Fx, Fy, Fz);
+        const float px = jx + 0.5f * Fx, py = jy + 0.5f * Fy, pz = jz + 0.5f * Fz;
+        acc[0] += widen(0.5f * (px * px + py * py + pz * pz) / (1.0f + drho));
+    });
+    block_sum(acc);
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        part[4 * blockIdx.x] = acc[0];
         part[4 * blockIdx.x + 1] = 0.0;
         part[4 * blockIdx.x + 2] = 0.0;
         part[4 * blockIdx.x + 3] = 0.0;
@@ -333,7 +322,7 @@ cudaError_t launch_energy_seed(const void *f, float *lam_out, float *gF, const S
     }
     g.gF = gF;
     const CellLaunch L = cell_launch(a.g);
-    energy_seed_kernel<Q, T><<<L.grid, L.block, 0, st>>>(static_cast<const T *>(f), a, g);
+    energy_seed_kernel<Q, T><<<L.grid, L.block, 0, st>>>(read_io<Q, T>(f, a.g), a, g);
     return cudaGetLastError();
 }
 
@@ -347,14 +336,14 @@ cudaError_t launch_macro_seed(const void *f, const float *g_rho, const float *g_
     }
     g.gF = gF;
     const CellLaunch L = cell_launch(a.g);
-    macro_seed_kernel<Q, T><<<L.grid, L.block, 0, st>>>(static_cast<const T *>(f), a, g, g_rho, g_u);
+    macro_seed_kernel<Q, T><<<L.grid, L.block, 0, st>>>(read_io<Q, T>(f, a.g), a, g, g_rho, g_u);
     return cudaGetLastError();
 }
 
 template <int Q, typename T>
-cudaError_t launch_energy(const void *f, const StepArgs &a, double *part, int blocks,
-                          cudaStream_t st) {
-    energy_kernel<Q, T><<<blocks, kRedThreads, 0, st>>>(static_cast<const T *>(f), a, part);
+cudaError_t launch_energy(const void *f, const StepArgs &a, double *part, cudaStream_t st) {
+    const RedLaunch L = red_launch(a.g);
+    energy_kernel<Q, T><<<L.blocks, L.block, 0, st>>>(read_io<Q, T>(f, a.g), a, part);
     return cudaGetLastError();
 }
 
@@ -366,7 +355,7 @@ cudaError_t launch_energy(const void *f, const StepArgs &a, double *part, int bl
     EXT template cudaError_t launch_macro_seed<Q, T>(const void *, const float *, const float *, \
                                                      float *, float *, const StepArgs &,        \
                                                      cudaStream_t);                             \
-    EXT template cudaError_t launch_energy<Q, T>(const void *, const StepArgs &, double *, int,  \
+    EXT template cudaError_t launch_energy<Q, T>(const void *, const StepArgs &, double *,       \
                                                  cudaStream_t);
 
 }  // namespace lbm

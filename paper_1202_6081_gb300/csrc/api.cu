@@ -154,9 +154,8 @@ struct MacroSeedFn {
 };
 template <int Q, typename T>
 struct EnergyFn {
-    static cudaError_t run(const void *f, const lbm::StepArgs &a, double *part, int blocks,
-                           cudaStream_t s) {
-        return lbm::launch_energy<Q, T>(f, a, part, blocks, s);
+    static cudaError_t run(const void *f, const lbm::StepArgs &a, double *part, cudaStream_t s) {
+        return lbm::launch_energy<Q, T>(f, a, part, s);
     }
 };
 
@@ -200,9 +199,9 @@ struct MacroFn {
 };
 template <int Q, typename T>
 struct ConsFn {
-    static cudaError_t run(const void *buf, const lbm::StepArgs &a, double *part, int blocks,
+    static cudaError_t run(const void *buf, const lbm::StepArgs &a, double *part,
                            cudaStream_t s) {
-        return lbm::launch_conservation<Q, T>(buf, a, part, blocks, s);
+        return lbm::launch_conservation<Q, T>(buf, a, part, s);
     }
 };
 
@@ -486,12 +485,12 @@ lbm_status lbm_conservation(lbm_ctx *c, double out[4], void *stream) {
     if (!c || !out) return LBM_EINVAL;
     if (!c->bound || !c->state_set) return LBM_ESTATE;
     const long long N = (long long)c->g.nx * c->g.ny * c->g.nz;
-    const int blocks = lbm::conservation_blocks(c->g);
+    const int blocks = lbm::red_launch(c->g).blocks;
     const lbm_status ms = ensure_scratch(c, blocks);
     if (ms != LBM_OK) return ms;
     const lbm::StepArgs a = step_args(c);
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = dispatch<ConsFn>(c, (const void *)c->buf[c->cur], a, c->red_scratch, blocks, s);
+    cudaError_t e = dispatch<ConsFn>(c, (const void *)c->buf[c->cur], a, c->red_scratch, s);
     if (e != cudaSuccess) return cuda_fail(c, e);
     double *tot = c->red_scratch + 4 * size_t(c->red_blocks);
     e = lbm::launch_reduce_final(c->red_scratch, blocks, tot, s);
@@ -605,11 +604,11 @@ lbm_status lbm_kinetic_energy(lbm_ctx *c, const void *f, double *out, void *stre
         a.g.layout = lbm::kPull;  // a caller's buffer holds a two-buffer state
     }
     if (!state_buffer_ok(f)) return LBM_EINVAL;
-    const int blocks = lbm::conservation_blocks(c->g);
+    const int blocks = lbm::red_launch(c->g).blocks;
     const lbm_status ms = ensure_scratch(c, blocks);
     if (ms != LBM_OK) return ms;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = dispatch<EnergyFn>(c, f, a, c->red_scratch, blocks, s);
+    cudaError_t e = dispatch<EnergyFn>(c, f, a, c->red_scratch, s);
     if (e != cudaSuccess) return cuda_fail(c, e);
     double *tot = c->red_scratch + 4 * size_t(c->red_blocks);
     e = lbm::launch_reduce_final(c->red_scratch, blocks, tot, s);
@@ -634,8 +633,8 @@ lbm_status lbm_kinetic_energy(lbm_ctx *c, const void *f, double *out, void *stre
 // that loads this library holds until the process exits.
 //
 // The array has room for one partial record (4 doubles) per (y, z) row of
-// the grid, for at most kNoAllocMaxRows rows (2 MiB).  Each call launches one
-// block per row, each block overwrites its own record, and the final
+// the grid, for at most kNoAllocMaxRows rows (2 MiB).  Each call launches at
+// most one block per row, each block overwrites its own record, and the final
 // reduction reads only the records this call wrote, so no part of the array
 // has to start at zero; it keeps the last call's contents.  Calls share the
 // array: two calls whose work overlaps on the GPU (different streams, or
@@ -713,9 +712,9 @@ lbm_status lbm_conservation_noalloc(lbm_ctx *c, double *out, void *stream) {
     if (st != LBM_OK) return st;
     const lbm::StepArgs a = step_args(c);
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = dispatch<ConsFn>(c, (const void *)c->buf[c->cur], a, part, int(rows), s);
+    cudaError_t e = dispatch<ConsFn>(c, (const void *)c->buf[c->cur], a, part, s);
     if (e != cudaSuccess) return cuda_fail(c, e);
-    e = lbm::launch_reduce_final(part, int(rows), dout, s);
+    e = lbm::launch_reduce_final(part, lbm::red_launch(c->g).blocks, dout, s);
     if (e != cudaSuccess) return cuda_fail(c, e);
     return LBM_OK;
 }

@@ -426,6 +426,171 @@ __device__ __forceinline__ f2 stored_pair(f2 v, float sc, const float4 &J) {
         return sc == 1.0f ? v : v * f2(sc);
 }
 
+// ---- one cell's distributions, for the kernels that read or load a state ----
+//
+// These kernels move a state once and compute little, so each access has to be
+// cheap: plane base pointers from the constant bank plus one 32-bit offset per
+// population (as in the step kernels), and the common case -- two-buffer
+// layout, no walls -- without the layout and wall selects.
+
+// Population q's stored value at plane + src -> deviation f - w; prod: the cell
+// whose collision produced it (the momentum reference of BF16 storage).
+template <int Q, typename T, int q>
+__device__ __forceinline__ float load_cell(const T *plane, int src, const float4 *ref, int prod,
+                                           bool wall) {
+    float v = Pair<T>::ld1(plane + src);
+    if constexpr (Storage<T>::kRef && has_ref<Q>(q)) {
+        const float r = ref_dot<Q, q>(load_ref<ey<Q>(q), ez<Q>(q)>(ref + (prod >> 1)));
+        v += wall ? -r : r;
+    }
+    return Storage<T>::kScaled ? v * float(weight<Q>(q)) : v;
+}
+
+// Pre-collision deviations f_alpha(x) - w_alpha of one cell (slot order).
+template <int Q, typename T>
+__device__ __forceinline__ void gather(const StepIO<T> &io, const Grid &g, int x, int y, int z,
+                                       float (&f)[Q]) {
+    const int xs[3] = {(x + 1 == g.nx) ? 0 : x + 1, x, (x == 0) ? g.nx - 1 : x - 1};
+    if (g.layout == kPull && g.bc == 0) {
+        const Rows<false> R = pull_rows<false>(g, y, z);
+        static_for<Q>([&](auto iq) {
+            constexpr int q = decltype(iq)::value;
+            const int src = R.off[ey<Q>(q) + 1][ez<Q>(q) + 1] + xs[ex<Q>(q) + 1];
+            f[q] = load_cell<Q, T, q>(io.in[q], src, io.ref_in, src, false);
+        });
+        return;
+    }
+    const Rows<true> R = pull_rows<true>(g, y, z);
+    const int own = R.own + x;
+    static_for<Q>([&](auto iq) {
+        constexpr int q = decltype(iq)::value;
+        constexpr int i = ex<Q>(q) + 1, j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
+        const bool wall = R.wall[j][k];
+        const int prod = wall ? own : R.off[j][k] + xs[i];
+        const bool opp = g.layout == kPull ? wall : g.layout == kAASwapped && !wall;
+        const T *plane = opp ? io.in[opposite<Q>(q)] : io.in[q];
+        f[q] = load_cell<Q, T, q>(plane, g.layout == kAANatural ? own : prod, io.ref_in, prod,
+                                  wall);
+    });
+}
+
+// Inverse of the pull: place the pre-collision values f_alpha(x) of one cell
+// where the next step will read them (the AA scheme loads into its natural
+// layout).  With momentum references (BF16) io.ref_out must already hold J of
+// every pair (ref_init_kernel), and each value is stored relative to the
+// reference of its producer, as a reader will add it back.
+template <int Q, typename T>
+__device__ __forceinline__ void scatter_state(const StepIO<T> &io, const Grid &g, int x, int y,
+                                              int z, const float (&f)[Q]) {
+    const int xs[3] = {(x + 1 == g.nx) ? 0 : x + 1, x, (x == 0) ? g.nx - 1 : x - 1};
+    const Rows<true> R = pull_rows<true>(g, y, z);
+    const int own = R.own + x;
+    static_for<Q>([&](auto iq) {
+        constexpr int q = decltype(iq)::value;
+        constexpr int i = ex<Q>(q) + 1, j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
+        const bool wall = R.wall[j][k];
+        const int prod = wall ? own : R.off[j][k] + xs[i];
+        float ref = 0.0f;
+        if constexpr (Storage<T>::kRef && has_ref<Q>(q)) {
+            const float r = ref_dot<Q, q>(load_ref<ey<Q>(q), ez<Q>(q)>(io.ref_out + (prod >> 1)));
+            ref = wall ? -r : r;
+        }
+        // opposite slots have equal weights
+        T *plane = g.layout == kPull && wall ? io.out[opposite<Q>(q)] : io.out[q];
+        store_dev<Q, T>(plane + (g.layout == kPull ? prod : own), q, f[q], ref);
+    });
+}
+
+// FP64 arithmetic of the state readers and writers, on the integer pipe.  GB300
+// issues about one FP64 operation per clock and SM (64-bit integer conversions
+// too), so one FP64 addition per population takes longer than the memory
+// traffic: 192^3 D3Q27 FP32, get_state 709 us and set_state 668 us with the
+// FP64 pipe 86-89 % busy, against 338 us of bytes.  The functions below return
+// the same bits; values outside their range take the FP64 instruction.
+
+// float -> double, exactly.
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u || m == 0u)  // normal or zero
+        return __hiloint2double(int((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)),
+                                int(b << 29));
+    return double(v);
+}
+
+// exponent of a weight: 2^e <= w < 2^(e + 1), and its mantissa w 2^(52 - e)
+__host__ __device__ constexpr int weight_exponent(double w) {
+    int e = 0;
+    while (w < 1.0) {
+        w *= 2.0;
+        --e;
+    }
+    return e;
+}
+__host__ __device__ constexpr long long weight_mantissa(double w) {
+    for (int i = weight_exponent(w); i < 52; ++i) w *= 2.0;
+    return (long long)w;
+}
+
+// w_q + v, rounded to nearest even.  In units of 2^(e - 52) both are integers
+// (|v| >= 2^(e - 29): 24 significant bits), their sum s is exact, and one of
+// three positions of its leading bit gives the result; only the highest one
+// drops a bit.  |v| < 2^(e - 54), zero included, leaves w.
+template <int Q, int q>
+__device__ __forceinline__ double weight_plus(float v) {
+    constexpr double w = weight<Q>(q);
+    constexpr int e = weight_exponent(w);
+    constexpr long long mw = weight_mantissa(w);
+    const unsigned b = __float_as_uint(v);
+    const int up = int(b >> 23 & 0xffu) - (127 + e - 29);
+    if (up < -25) return w;
+    if (up >= 0 && up <= 30) {
+        const long long m = (long long)((b & 0x7fffffu) | 0x800000u) << up;
+        const unsigned long long s = (unsigned long long)(int(b) < 0 ? mw - m : mw + m);
+        const unsigned top = unsigned(s >> 51);
+        if (top - 1u < 7u) {  // 2^51 <= s < 2^54
+            unsigned long long r = s;
+            int er = e;
+            if (top == 1u) {
+                r = s << 1;
+                er = e - 1;
+            } else if (top >= 4u) {
+                r = (s + (s >> 1 & 1u)) >> 1;
+                er = e + 1;
+            }
+            return __longlong_as_double((long long)r + ((long long)(1022 + er) << 52));
+        }
+    }
+    return w + double(v);
+}
+
+// float(f - w_q): the exact difference, rounded once to nearest even.  For f in
+// w's binade or a neighbouring one both are integers in units of 2^(e - 53), and
+// a difference below 2^53 is what the FP64 subtraction gives exactly.  It is
+// shifted into 32 bits, what falls off kept as a sticky bit, and converted.
+template <int Q, int q>
+__device__ __forceinline__ float deviation(double f) {
+    constexpr double w = weight<Q>(q);
+    constexpr int e = weight_exponent(w);
+    constexpr long long mw = 2 * weight_mantissa(w);
+    const unsigned hi = unsigned(__double2hiint(f));
+    const unsigned up = (hi >> 20) - unsigned(1023 + e - 1);
+    if (up <= 2u) {
+        const unsigned long long m =
+            (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | unsigned(__double2loint(f));
+        const long long d = (long long)(m << up) - mw;
+        const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
+        const unsigned ah = unsigned(a >> 32), al = unsigned(a);
+        if (ah < 1u << 21) {
+            const int n = 32 - __clz(int(ah));
+            unsigned t = __funnelshift_r(al, ah, n);
+            if (al & ((1u << n) - 1u)) t |= 1u;
+            const float r = __uint2float_rn(t) * __uint_as_float(unsigned(127 + e - 53 + n) << 23);
+            return d < 0 ? -r : r;
+        }
+    }
+    return float(f - w);
+}
+
 // One fused step, one cell per thread: pull-gather (streaming with
 // bounce-back), collision, store.  With BF16 momentum references the cells
 // x (even) and x + 1, held by neighbouring lanes, exchange their velocities
@@ -812,7 +977,7 @@ __global__ void __launch_bounds__(128, (kAAOddBlocks<Q, T, kForce>))
 
 // Initial state from FP64 density and velocity fields.
 template <int Q, typename T>
-__global__ void __launch_bounds__(128) init_kernel(T *__restrict__ buf, const StepArgs a,
+__global__ void __launch_bounds__(128) init_kernel(const StepIO<T> io, const StepArgs a,
                                                    const double *__restrict__ rho,
                                                    const double *__restrict__ u) {
     int x, y, z;
@@ -824,21 +989,23 @@ __global__ void __launch_bounds__(128) init_kernel(T *__restrict__ buf, const St
     float f[Q];
     equilibrium<Q>(float(rho[c] - 1.0), float(u[c]), float(u[N + c]), float(u[2 * N + c]), Fx, Fy,
                    Fz, f);
-    scatter_state<Q, T>(buf, a.g, pull_sources(a.g, x, y, z), f);
+    scatter_state<Q, T>(io, a.g, x, y, z, f);
 }
 
 // Load a dense FP64 state [Q][N] (pre-collision values at their own cells).
 template <int Q, typename T>
-__global__ void __launch_bounds__(128) set_state_kernel(T *__restrict__ buf, const Grid g,
+__global__ void __launch_bounds__(128) set_state_kernel(const StepIO<T> io, const Grid g,
                                                         const double *__restrict__ fin) {
     int x, y, z;
     if (!cell_coords(g, x, y, z)) return;
     const long long N = (long long)g.nx * g.ny * g.nz;
-    const long long c = dense_index(g, x, y, z);
+    const double *src = fin + dense_index(g, x, y, z);
     float f[Q];
-#pragma unroll
-    for (int a = 0; a < Q; ++a) f[a] = float(fin[a * N + c] - weight<Q>(a));
-    scatter_state<Q, T>(buf, g, pull_sources(g, x, y, z), f);
+    static_for<Q>([&](auto iq) {
+        constexpr int q = decltype(iq)::value;
+        f[q] = deviation<Q, q>(__ldcs(src + q * N));
+    });
+    scatter_state<Q, T>(io, g, x, y, z, f);
 }
 
 // BF16 momentum references of a state being loaded (reference array 0), one
@@ -882,16 +1049,18 @@ __global__ void __launch_bounds__(128) ref_init_kernel(T *__restrict__ buf, cons
 
 // Read the state back as dense FP64 [Q][N].
 template <int Q, typename T>
-__global__ void __launch_bounds__(128) get_state_kernel(const T *__restrict__ buf, const Grid g,
+__global__ void __launch_bounds__(128) get_state_kernel(const StepIO<T> io, const Grid g,
                                                         double *__restrict__ fout) {
     int x, y, z;
     if (!cell_coords(g, x, y, z)) return;
     const long long N = (long long)g.nx * g.ny * g.nz;
-    const long long c = dense_index(g, x, y, z);
+    double *dst = fout + dense_index(g, x, y, z);
     float f[Q];
-    gather<Q, T>(buf, g, pull_sources(g, x, y, z), f);
-#pragma unroll
-    for (int a = 0; a < Q; ++a) fout[a * N + c] = weight<Q>(a) + double(f[a]);
+    gather<Q, T>(io, g, x, y, z, f);
+    static_for<Q>([&](auto iq) {
+        constexpr int q = decltype(iq)::value;
+        __stcs(dst + q * N, weight_plus<Q, q>(f[q]));
+    });
 }
 
 template <int Q>
@@ -909,7 +1078,7 @@ __device__ __forceinline__ void moments(const float (&f)[Q], float &drho, float 
 
 // Density and velocity (Eqs. densitycalculation, velocitycalculation).
 template <int Q, typename T>
-__global__ void __launch_bounds__(128) macro_kernel(const T *__restrict__ buf, const StepArgs a,
+__global__ void __launch_bounds__(128) macro_kernel(const StepIO<T> io, const StepArgs a,
                                                     float *__restrict__ rho,
                                                     float *__restrict__ u) {
     int x, y, z;
@@ -917,7 +1086,7 @@ __global__ void __launch_bounds__(128) macro_kernel(const T *__restrict__ buf, c
     const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
     const long long c = dense_index(a.g, x, y, z);
     float f[Q];
-    gather<Q, T>(buf, a.g, pull_sources(a.g, x, y, z), f);
+    gather<Q, T>(io, a.g, x, y, z, f);
     float drho, jx, jy, jz, Fx, Fy, Fz;
     moments<Q>(f, drho, jx, jy, jz);
     cell_force(a, c, N, Fx, Fy, Fz);
@@ -930,48 +1099,80 @@ __global__ void __launch_bounds__(128) macro_kernel(const T *__restrict__ buf, c
     }
 }
 
-constexpr int kRedThreads = 256;
-constexpr int kRedMaxBlocks = 2048;
+// Global sums.  Blocks of at most 128 threads, shaped like the other per-cell
+// kernels' (short rows share a block), stride over the rows of the grid, at
+// most eight blocks per SM resident; each leaves one partial record of 4
+// doubles, added up in a fixed order by reduce_final_kernel.  A cell's moments
+// are FP32 sums of its stored deviations; the running sums across cells are
+// FP64.
+constexpr int kFinalThreads = 256;
+constexpr int kRedBlocks = 152 * 8;
 
-// Partial sums of (rho - 1, rho u) per block, fixed order.  Each block takes
-// whole (y, z) rows (row = blockIdx.x + k * gridDim.x) and its threads stride
-// along x, so cells are decoded with one division per row.  A cell's moments
-// are FP32 sums of its 27 (15) stored deviations; the running sums across
-// cells are FP64 (FP64 is slow on this GPU, so it is kept to 4 adds per cell).
-template <int Q, typename T>
-__global__ void __launch_bounds__(kRedThreads) conservation_kernel(const T *__restrict__ buf,
-                                                                   const StepArgs a,
-                                                                   double *__restrict__ part) {
-    const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
-    const long long rows = (long long)a.g.ny * a.g.nz;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-        const int y = int(row % a.g.ny), z = int(row / a.g.ny);
-        for (int x = threadIdx.x; x < a.g.nx; x += blockDim.x) {
-            float f[Q];
-            gather<Q, T>(buf, a.g, pull_sources(a.g, x, y, z), f);
-            float drho, jx, jy, jz, Fx, Fy, Fz;
-            moments<Q>(f, drho, jx, jy, jz);
-            cell_force(a, row * a.g.nx + x, N, Fx, Fy, Fz);
-            acc[0] += double(drho);
-            acc[1] += double(jx + 0.5f * Fx);
-            acc[2] += double(jy + 0.5f * Fy);
-            acc[3] += double(jz + 0.5f * Fz);
-        }
+struct RedLaunch {
+    dim3 block;
+    int blocks;
+};
+inline RedLaunch red_launch(const Grid &g) {
+    RedLaunch L;
+    L.block = cell_launch(g).block;
+    const long long groups = ((long long)g.ny * g.nz + L.block.y - 1) / L.block.y;
+    L.blocks = int(groups < kRedBlocks ? groups : kRedBlocks);
+    return L;
+}
+
+// fn(x, y, z, dense cell index) over the block's share of the cells.
+template <typename Fn>
+__device__ __forceinline__ void for_cells(const Grid &g, Fn &&fn) {
+    const unsigned rows = unsigned(g.ny) * unsigned(g.nz);  // ny, nz <= 65535
+    for (unsigned row = blockIdx.x * blockDim.y + threadIdx.y; row < rows;
+         row += gridDim.x * blockDim.y) {
+        const int z = int(row / unsigned(g.ny)), y = int(row - unsigned(z) * unsigned(g.ny));
+        for (int x = threadIdx.x; x < g.nx; x += blockDim.x)
+            fn(x, y, z, (long long)row * g.nx + x);
     }
-    __shared__ double sh[4][kRedThreads];
+}
+
+// Sum of the threads' acc[K] over the block (whole warps, at most four), in a
+// fixed order; valid in thread 0.
+template <int K>
+__device__ __forceinline__ void block_sum(double (&acc)[K]) {
+    __shared__ double sh[K][4];
+    const int t = threadIdx.y * blockDim.x + threadIdx.x;
+    const int warps = int(blockDim.x * blockDim.y) >> 5;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] = acc[k];
+    for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], d);
+        if ((t & 31) == 0) sh[k][t >> 5] = acc[k];
+    }
     __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
+    if (t == 0)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
+        for (int k = 0; k < K; ++k)
+            for (int w = 1; w < warps; ++w) acc[k] += sh[k][w];
+}
+
+// Partial sums of (rho - 1, rho u).
+template <int Q, typename T>
+__global__ void __launch_bounds__(128, 8) conservation_kernel(const StepIO<T> io, const StepArgs a,
+                                                              double *__restrict__ part) {
+    const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for_cells(a.g, [&](int x, int y, int z, long long c) {
+        float f[Q];
+        gather<Q, T>(io, a.g, x, y, z, f);
+        float drho, jx, jy, jz, Fx, Fy, Fz;
+        moments<Q>(f, drho, jx, jy, jz);
+        cell_force(a, c, N, Fx, Fy, Fz);
+        acc[0] += widen(drho);
+        acc[1] += widen(jx + 0.5f * Fx);
+        acc[2] += widen(jy + 0.5f * Fy);
+        acc[3] += widen(jz + 0.5f * Fz);
+    });
+    block_sum(acc);
+    if (threadIdx.x == 0 && threadIdx.y == 0)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) part[4 * blockIdx.x + k] = sh[k][0];
+        for (int k = 0; k < 4; ++k) part[4 * blockIdx.x + k] = acc[k];
 }
 
 // Launchers.  The kernels_q27_*.cu and kernels_q15.cu units hold their
@@ -1011,17 +1212,31 @@ inline bool higher_rates_are_one(const StepArgs &a) {
     return true;
 }
 
+// Plane pointers of an input and an output state buffer (either may be null:
+// not accessed by the kernel then) and their BF16 reference arrays.
+template <int Q, typename T>
+StepIO<T> step_io(const void *fin, void *fout, const Grid &g, int ref_in = 0, int ref_out = 0) {
+    StepIO<T> io{};
+    for (int q = 0; q < Q; ++q) {
+        if (fin) io.in[q] = static_cast<const T *>(fin) + q * g.pop;
+        if (fout) io.out[q] = static_cast<T *>(fout) + q * g.pop;
+    }
+    if (Storage<T>::kRef && fin)
+        io.ref_in = ref_array<Q>(static_cast<const T *>(fin), g.pop, ref_in);
+    if (Storage<T>::kRef && fout) io.ref_out = ref_array<Q>(static_cast<T *>(fout), g.pop, ref_out);
+    return io;
+}
+// The same for a kernel that only reads the state, in whichever layout.
+template <int Q, typename T>
+StepIO<T> read_io(const void *f, const Grid &g) {
+    return step_io<Q, T>(f, nullptr, g, g.layout == kAASwapped ? 1 : 0);
+}
+
 // The two-cells-per-thread kernels serve grids with even nx (D3Q27 and
 // D3Q15); odd nx takes the one-cell kernel.
 template <int Q, typename T>
 cudaError_t launch_step(const void *fin, void *fout, const StepArgs &a, cudaStream_t st) {
-    StepIO<T> io;
-    for (int q = 0; q < 27; ++q) {
-        io.in[q] = static_cast<const T *>(fin) + (q < Q ? q * a.g.pop : 0);
-        io.out[q] = static_cast<T *>(fout) + (q < Q ? q * a.g.pop : 0);
-    }
-    io.ref_in = Storage<T>::kRef ? ref_array<Q>(static_cast<const T *>(fin), a.g.pop, 0) : nullptr;
-    io.ref_out = Storage<T>::kRef ? ref_array<Q>(static_cast<T *>(fout), a.g.pop, 0) : nullptr;
+    const StepIO<T> io = step_io<Q, T>(fin, fout, a.g);
     const bool walls = a.g.bc != 0;
     if constexpr (std::is_same<T, float>::value) {
         if (a.sr32) {  // stochastically rounded FP32 update: the one-cell kernel, any nx
@@ -1096,16 +1311,8 @@ void launch_aa_kernels(const StepIO<T> &io, const StepArgs &a, const PackedRates
 // no force.
 template <int Q, typename T>
 cudaError_t launch_step_aa(void *buf, const StepArgs &a, bool even, cudaStream_t st) {
-    StepIO<T> io;
-    for (int q = 0; q < 27; ++q) {
-        io.in[q] = static_cast<const T *>(buf) + (q < Q ? q * a.g.pop : 0);
-        io.out[q] = static_cast<T *>(buf) + (q < Q ? q * a.g.pop : 0);
-    }
     // BF16 references: array 0 for the natural layout, 1 for the swapped one
-    io.ref_in = Storage<T>::kRef ? ref_array<Q>(static_cast<const T *>(buf), a.g.pop, even ? 0 : 1)
-                                 : nullptr;
-    io.ref_out = Storage<T>::kRef ? ref_array<Q>(static_cast<T *>(buf), a.g.pop, even ? 1 : 0)
-                                  : nullptr;
+    const StepIO<T> io = step_io<Q, T>(buf, buf, a.g, even ? 0 : 1, even ? 1 : 0);
     Grid half = a.g;
     half.nx = a.g.nx / 2;
     const CellLaunch L = cell_launch(half);
@@ -1143,7 +1350,7 @@ cudaError_t launch_init(void *buf, const StepArgs &a, const double *rho, const d
         if (e != cudaSuccess) return e;
     }
     const CellLaunch L = cell_launch(a.g);
-    init_kernel<Q, T><<<L.grid, L.block, 0, st>>>(static_cast<T *>(buf), a, rho, u);
+    init_kernel<Q, T><<<L.grid, L.block, 0, st>>>(step_io<Q, T>(nullptr, buf, a.g), a, rho, u);
     return cudaGetLastError();
 }
 
@@ -1154,14 +1361,14 @@ cudaError_t launch_set_state(void *buf, const Grid &g, const double *f, cudaStre
         if (e != cudaSuccess) return e;
     }
     const CellLaunch L = cell_launch(g);
-    set_state_kernel<Q, T><<<L.grid, L.block, 0, st>>>(static_cast<T *>(buf), g, f);
+    set_state_kernel<Q, T><<<L.grid, L.block, 0, st>>>(step_io<Q, T>(nullptr, buf, g), g, f);
     return cudaGetLastError();
 }
 
 template <int Q, typename T>
 cudaError_t launch_get_state(const void *buf, const Grid &g, double *f, cudaStream_t st) {
     const CellLaunch L = cell_launch(g);
-    get_state_kernel<Q, T><<<L.grid, L.block, 0, st>>>(static_cast<const T *>(buf), g, f);
+    get_state_kernel<Q, T><<<L.grid, L.block, 0, st>>>(read_io<Q, T>(buf, g), g, f);
     return cudaGetLastError();
 }
 
@@ -1169,29 +1376,21 @@ template <int Q, typename T>
 cudaError_t launch_macro(const void *buf, const StepArgs &a, float *rho, float *u,
                          cudaStream_t st) {
     const CellLaunch L = cell_launch(a.g);
-    macro_kernel<Q, T><<<L.grid, L.block, 0, st>>>(static_cast<const T *>(buf), a, rho, u);
+    macro_kernel<Q, T><<<L.grid, L.block, 0, st>>>(read_io<Q, T>(buf, a.g), a, rho, u);
     return cudaGetLastError();
 }
 
+// Partial records of the conservation sums: red_launch(g).blocks of them.
 template <int Q, typename T>
-cudaError_t launch_conservation(const void *buf, const StepArgs &a, double *part, int blocks,
+cudaError_t launch_conservation(const void *buf, const StepArgs &a, double *part,
                                 cudaStream_t st) {
-    conservation_kernel<Q, T><<<blocks, kRedThreads, 0, st>>>(static_cast<const T *>(buf), a,
-                                                              part);
+    const RedLaunch L = red_launch(a.g);
+    conservation_kernel<Q, T><<<L.blocks, L.block, 0, st>>>(read_io<Q, T>(buf, a.g), a, part);
     return cudaGetLastError();
 }
 
 // Final reduction of the per-block partials to 4 doubles (one block).
 cudaError_t launch_reduce_final(const double *part, int blocks, double *out, cudaStream_t st);
-
-// Number of partial-sum blocks the conservation reduction uses: one per
-// (y, z) row up to kRedMaxBlocks.
-inline int conservation_blocks(const Grid &g) {
-    long long b = (long long)g.ny * g.nz;
-    if (b > kRedMaxBlocks) b = kRedMaxBlocks;
-    if (b < 1) b = 1;
-    return int(b);
-}
 
 #define LBM_INSTANTIATE_1(EXT, Q, T)                                                             \
     EXT template cudaError_t launch_step<Q, T>(const void *, void *, const StepArgs &,          \
@@ -1206,7 +1405,7 @@ inline int conservation_blocks(const Grid &g) {
     EXT template cudaError_t launch_macro<Q, T>(const void *, const StepArgs &, float *, float *, \
                                                 cudaStream_t);                                 \
     EXT template cudaError_t launch_conservation<Q, T>(const void *, const StepArgs &, double *, \
-                                                       int, cudaStream_t);
+                                                       cudaStream_t);
 
 #define LBM_INSTANTIATE(EXT, Q)                \
     LBM_INSTANTIATE_1(EXT, Q, float)           \

@@ -5,18 +5,18 @@
 namespace lbm {
 LBM_INSTANTIATE(, 15)
 
-__global__ void __launch_bounds__(kRedThreads) reduce_final_kernel(const double *__restrict__ part,
+__global__ void __launch_bounds__(kFinalThreads) reduce_final_kernel(const double *__restrict__ part,
                                                                    int blocks,
                                                                    double *__restrict__ out) {
-    __shared__ double sh[4][kRedThreads];
+    __shared__ double sh[4][kFinalThreads];
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < blocks; b += kRedThreads)
+    for (int b = threadIdx.x; b < blocks; b += kFinalThreads)
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[k] += part[4 * b + k];
 #pragma unroll
     for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] = acc[k];
     __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
+    for (int w = kFinalThreads / 2; w > 0; w >>= 1) {
         if (threadIdx.x < w)
 #pragma unroll
             for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + w];
@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(kRedThreads) reduce_final_kernel(const double 
 }
 
 cudaError_t launch_reduce_final(const double *part, int blocks, double *out, cudaStream_t st) {
-    reduce_final_kernel<<<1, kRedThreads, 0, st>>>(part, blocks, out);
+    reduce_final_kernel<<<1, kFinalThreads, 0, st>>>(part, blocks, out);
     return cudaGetLastError();
 }
 }  // namespace lbm

@@ -320,110 +320,4 @@ __host__ __device__ inline float4 *ref_array(T *buf, long long pop, int which) {
     return reinterpret_cast<float4 *>(buf + (long long)Q * pop) + (long long)which * (pop / 2);
 }
 
-// Source coordinates of the pull for one cell.  Index 0, 1, 2 of each array
-// is the velocity component -1, 0, +1; the source along an axis is the cell
-// coordinate minus the component.  wall[...] is set where that source lies
-// beyond a bounce-back wall.
-struct PullSources {
-    int xs[3];
-    long long row[3][3];  // (zs * ny + ys) * px for (cy, cz)
-    bool wall[3][3];      // bounce back for (cy, cz)
-    long long own;        // (z * ny + y) * px + x
-};
-
-__device__ __forceinline__ PullSources pull_sources(const Grid &g, int x, int y, int z) {
-    PullSources s;
-    s.xs[0] = (x + 1 == g.nx) ? 0 : x + 1;
-    s.xs[1] = x;
-    s.xs[2] = (x == 0) ? g.nx - 1 : x - 1;
-    int ys[3], zs[3];
-    bool wy[3], wz[3];
-    ys[1] = y;
-    wy[1] = false;
-    ys[0] = (y + 1 == g.ny) ? 0 : y + 1;
-    wy[0] = (y + 1 == g.ny) && (g.bc & kWallY);
-    ys[2] = (y == 0) ? g.ny - 1 : y - 1;
-    wy[2] = (y == 0) && (g.bc & kWallY);
-    zs[1] = z;
-    wz[1] = false;
-    zs[0] = (z + 1 == g.nz) ? 0 : z + 1;
-    wz[0] = (z + 1 == g.nz) && (g.bc & kWallZ);
-    zs[2] = (z == 0) ? g.nz - 1 : z - 1;
-    wz[2] = (z == 0) && (g.bc & kWallZ);
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            s.row[j][k] = ((long long)zs[k] * g.ny + ys[j]) * g.px;
-            s.wall[j][k] = wy[j] || wz[k];
-        }
-    s.own = ((long long)z * g.ny + y) * g.px + x;
-    return s;
-}
-
-// Pre-collision deviations f_alpha(x) - w_alpha of one cell (slot order).
-template <int Q, typename T>
-__device__ __forceinline__ void gather(const T *__restrict__ fin, const Grid &g,
-                                       const PullSources &s, float (&f)[Q]) {
-#pragma unroll
-    for (int a = 0; a < Q; ++a) {
-        const int j = ey<Q>(a) + 1, k = ez<Q>(a) + 1, i = ex<Q>(a) + 1;
-        const int o = opposite<Q>(a);
-        long long idx;
-        if (g.layout == kAANatural) {
-            idx = (long long)a * g.pop + s.own;
-        } else if (s.wall[j][k]) {
-            idx = (long long)(g.layout == kPull ? o : a) * g.pop + s.own;
-        } else {
-            idx = (long long)(g.layout == kPull ? a : o) * g.pop + s.row[j][k] + s.xs[i];
-        }
-        float v = Storage<T>::load(fin + idx);
-        if constexpr (Storage<T>::kRef) {
-            if (has_ref<Q>(a)) {
-                // producer: x - e_a, or x itself behind a wall (population opp(a))
-                const float4 *R = ref_array<Q>(fin, g.pop, g.layout == kAASwapped ? 1 : 0);
-                const long long prod = s.wall[j][k] ? s.own : s.row[j][k] + s.xs[i];
-                const float4 J = __ldg(R + (prod >> 1));
-                const float r = ex<Q>(a) * J.x + ey<Q>(a) * J.y + ez<Q>(a) * J.z;
-                v += s.wall[j][k] ? -r : r;
-            }
-        }
-        // the weight of a slot and of its opposite are equal
-        f[a] = Storage<T>::kScaled ? v * float(weight<Q>(a)) : v;
-    }
-}
-
-// Inverse of the pull: place the pre-collision values f_alpha(x) of one cell
-// where the next step will read them (used to load a state; the AA scheme
-// loads into its natural layout).
-// With momentum references (BF16) the reference array 0 must already hold J
-// of every pair (ref_init_kernel), and each value is stored relative to the
-// reference of its producer, as a reader will add it back.
-template <int Q, typename T>
-__device__ __forceinline__ void scatter_state(T *__restrict__ buf, const Grid &g,
-                                              const PullSources &s, const float (&f)[Q]) {
-#pragma unroll
-    for (int a = 0; a < Q; ++a) {
-        const int j = ey<Q>(a) + 1, k = ez<Q>(a) + 1, i = ex<Q>(a) + 1;
-        float ref = 0.0f;
-        if constexpr (Storage<T>::kRef) {
-            if (has_ref<Q>(a)) {
-                const float4 *R = ref_array<Q>(static_cast<const T *>(buf), g.pop, 0);
-                const long long prod = s.wall[j][k] ? s.own : s.row[j][k] + s.xs[i];
-                const float4 J = R[prod >> 1];
-                const float r = ex<Q>(a) * J.x + ey<Q>(a) * J.y + ez<Q>(a) * J.z;
-                ref = s.wall[j][k] ? -r : r;
-            }
-        }
-        if (g.layout != kPull) {
-            store_dev<Q, T>(buf + (long long)a * g.pop + s.own, a, f[a], ref);
-        } else if (s.wall[j][k]) {
-            const int o = opposite<Q>(a);
-            store_dev<Q, T>(buf + (long long)o * g.pop + s.own, o, f[a], ref);
-        } else {
-            store_dev<Q, T>(buf + (long long)a * g.pop + s.row[j][k] + s.xs[i], a, f[a], ref);
-        }
-    }
-}
-
 }  // namespace lbm
