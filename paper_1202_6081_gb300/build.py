@@ -1,8 +1,8 @@
 """Build liblbm.so, the C-ABI CUDA library, in-tree for sm_103a.
 
-Each translation unit under csrc/ is compiled by nvcc in parallel, then
-linked into paper_1202_6081_gb300/liblbm.so (CUDA runtime linked
-statically).  Run ``python -m paper_1202_6081_gb300.build`` or call
+The translation units (csrc/kernels.cu once per lattice, storage type and
+group of kernels) are compiled by nvcc in parallel, then linked into
+paper_1202_6081_gb300/liblbm.so (CUDA runtime linked statically).  Run ``python -m paper_1202_6081_gb300.build`` or call
 ``build()``.
 """
 from __future__ import annotations
@@ -19,8 +19,12 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblbm.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["kernels_q27_f32.cu", "kernels_q27_f16.cu", "kernels_q27_bf16.cu", "kernels_q15.cu",
-           "kernels_q15_adjoint.cu", "api.cu"]
+# translation units: (object name, source, macro definitions); the slowest first
+UNITS = [("kernels_%s_q%d_%s" % (group.lower(), Q, name), "kernels.cu",
+          ["-DLBM_GROUP=" + group, "-DLBM_Q=%d" % Q, "-DLBM_T=" + T])
+         for group in ("STEP", "ADJOINT", "INPLACE", "STATE") for Q in (27, 15)
+         for name, T in (("f32", "float"), ("f16", "__half"), ("bf16", "__nv_bfloat16"))]
+UNITS += [("reduce", "reduce.cu", []), ("api", "api.cu", [])]
 
 
 def nvcc() -> str:
@@ -56,16 +60,17 @@ def build(force: bool = False, verbose_ptxas: bool = False, quiet: bool = True) 
     cc = nvcc()
     flags = _flags(verbose_ptxas)
 
-    def compile_one(src):
-        obj = os.path.join(BUILD, os.path.splitext(src)[0] + ".o")
-        cmd = [cc, "-c", os.path.join(CSRC, src), "-o", obj] + flags
+    def compile_one(unit):
+        name, src, defines = unit
+        obj = os.path.join(BUILD, name + ".o")
+        cmd = [cc, "-c", os.path.join(CSRC, src), "-o", obj] + defines + flags
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
-            raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, r.stdout, r.stderr))
+            raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (name, r.stdout, r.stderr))
         return obj, r.stderr
 
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        results = list(ex.map(compile_one, SOURCES))
+    with ThreadPoolExecutor(max_workers=os.cpu_count() or 4) as ex:
+        results = list(ex.map(compile_one, UNITS))
     objs = [o for o, _ in results]
     if verbose_ptxas or not quiet:
         for _, log in results:

@@ -9,14 +9,17 @@
 #include "adjoint_kernels.cuh"
 
 namespace lbm {
-LBM_INSTANTIATE(extern, 27)
-LBM_INSTANTIATE(extern, 15)
-LBM_INSTANTIATE_ADJOINT(extern, 27, float)
-LBM_INSTANTIATE_ADJOINT(extern, 15, float)
-LBM_INSTANTIATE_ADJOINT(extern, 27, __half)
-LBM_INSTANTIATE_ADJOINT(extern, 15, __half)
-LBM_INSTANTIATE_ADJOINT(extern, 27, __nv_bfloat16)
-LBM_INSTANTIATE_ADJOINT(extern, 15, __nv_bfloat16)
+#define LBM_EXTERN(Q, T)                \
+    LBM_INSTANTIATE_STEP(extern, Q, T)    \
+    LBM_INSTANTIATE_INPLACE(extern, Q, T) \
+    LBM_INSTANTIATE_STATE(extern, Q, T)   \
+    LBM_INSTANTIATE_ADJOINT(extern, Q, T)
+LBM_EXTERN(27, float)
+LBM_EXTERN(27, __half)
+LBM_EXTERN(27, __nv_bfloat16)
+LBM_EXTERN(15, float)
+LBM_EXTERN(15, __half)
+LBM_EXTERN(15, __nv_bfloat16)
 }  // namespace lbm
 
 // A captured run of steps (a CUDA graph), valid for the launch arguments,

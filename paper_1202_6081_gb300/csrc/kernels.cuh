@@ -1,7 +1,6 @@
 // Kernels of liblbm.so, templated over the lattice (Q = 27 or 15) and the
-// storage type (float, __half, __nv_bfloat16).  kernels_q27_f32.cu,
-// kernels_q27_f16.cu, kernels_q27_bf16.cu and kernels_q15.cu instantiate
-// them; api.cu calls the launchers.
+// storage type (float, __half, __nv_bfloat16).  kernels.cu instantiates the
+// launchers; api.cu calls them.
 #pragma once
 
 #include "collide_q15.cuh"
@@ -1175,9 +1174,8 @@ __global__ void __launch_bounds__(128, 8) conservation_kernel(const StepIO<T> io
         for (int k = 0; k < 4; ++k) part[4 * blockIdx.x + k] = acc[k];
 }
 
-// Launchers.  The kernels_q27_*.cu and kernels_q15.cu units hold their
-// explicit instantiations; api.cu sees them through the extern declarations
-// below.
+// Launchers.  kernels.cu holds their explicit instantiations; api.cu sees them
+// through extern declarations (the macros below).
 inline unsigned long long splat_bits(float v) {
     unsigned int u;
     memcpy(&u, &v, 4);
@@ -1392,10 +1390,13 @@ cudaError_t launch_conservation(const void *buf, const StepArgs &a, double *part
 // Final reduction of the per-block partials to 4 doubles (one block).
 cudaError_t launch_reduce_final(const double *part, int blocks, double *out, cudaStream_t st);
 
-#define LBM_INSTANTIATE_1(EXT, Q, T)                                                             \
-    EXT template cudaError_t launch_step<Q, T>(const void *, void *, const StepArgs &,          \
-                                               cudaStream_t);                                  \
-    EXT template cudaError_t launch_step_aa<Q, T>(void *, const StepArgs &, bool, cudaStream_t);  \
+#define LBM_INSTANTIATE_STEP(EXT, Q, T) \
+    EXT template cudaError_t launch_step<Q, T>(const void *, void *, const StepArgs &, cudaStream_t);
+
+#define LBM_INSTANTIATE_INPLACE(EXT, Q, T) \
+    EXT template cudaError_t launch_step_aa<Q, T>(void *, const StepArgs &, bool, cudaStream_t);
+
+#define LBM_INSTANTIATE_STATE(EXT, Q, T)                                                         \
     EXT template cudaError_t launch_init<Q, T>(void *, const StepArgs &, const double *,         \
                                                const double *, cudaStream_t);                  \
     EXT template cudaError_t launch_set_state<Q, T>(void *, const Grid &, const double *,        \
@@ -1406,10 +1407,5 @@ cudaError_t launch_reduce_final(const double *part, int blocks, double *out, cud
                                                 cudaStream_t);                                 \
     EXT template cudaError_t launch_conservation<Q, T>(const void *, const StepArgs &, double *, \
                                                        cudaStream_t);
-
-#define LBM_INSTANTIATE(EXT, Q)                \
-    LBM_INSTANTIATE_1(EXT, Q, float)           \
-    LBM_INSTANTIATE_1(EXT, Q, __half)          \
-    LBM_INSTANTIATE_1(EXT, Q, __nv_bfloat16)
 
 }  // namespace lbm

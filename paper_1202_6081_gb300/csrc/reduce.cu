@@ -1,10 +1,7 @@
-// Explicit instantiations of the D3Q15 kernels (FP32, FP16, BF16 storage)
-// and the final conservation reduction.
+// The final step of the global sums.
 #include "kernels.cuh"
 
 namespace lbm {
-LBM_INSTANTIATE(, 15)
-
 __global__ void __launch_bounds__(kFinalThreads) reduce_final_kernel(const double *__restrict__ part,
                                                                    int blocks,
                                                                    double *__restrict__ out) {
