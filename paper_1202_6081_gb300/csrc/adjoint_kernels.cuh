@@ -58,90 +58,47 @@ struct AdjointArgs {
     float *gF;                  // dense [3][N] accumulator or nullptr
 };
 
-template <int Q, typename T, bool kWalls>
-__global__ void __launch_bounds__(128) adjoint_kernel(const StepIO<T> io, const AdjointArgs g,
-                                                      const StepArgs a) {
-    int x, y, z;
-    if (!cell_coords(a.g, x, y, z)) return;
-    const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
-    const int xs[3] = {(x + 1 == a.g.nx) ? 0 : x + 1, x, (x == 0) ? a.g.nx - 1 : x - 1};
-    float f[Q], mu[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const int i = ex<Q>(q) + 1, j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
-        // state at t: pull from x - e_q
-        const bool wall = kWalls && R.wall[j][k];
-        const int src = wall ? R.own + x : R.off[j][k] + xs[i];
-        const T *plane = wall ? io.in[opposite<Q>(q)] : io.in[q];
-        float v = Storage<T>::load(plane + src);
-        if (Storage<T>::kRef && has_ref<Q>(q)) {  // BF16 momentum reference (lattice.cuh)
-            const float4 J = __ldg(io.ref_in + (src >> 1));
-            const float r = ex<Q>(q) * J.x + ey<Q>(q) * J.y + ez<Q>(q) * J.z;
-            v += wall ? -r : r;
+// The pair's adjoints of its post-collision values, from the mirrored
+// neighbours; kSel: with the wall selects.
+template <int Q, bool kSel, bool kWalls, bool kRag>
+__device__ __forceinline__ void pull_adjoint(const AdjointArgs &g, const Rows<kWalls> &R,
+                                             const PairCols<kRag> &X, f2 (&mu)[Q]) {
+    static_for<Q>([&](auto iq) {
+        constexpr int q = decltype(iq)::value;
+        constexpr int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
+        if (kSel && R.wall[2 - j][2 - k]) {
+            mu[q] = Pair<float>::ld2(element<kRag>(g.lam_next[opposite<Q>(q)], R.own + X.x0));
+        } else {
+            mu[q] = ld_shifted(g.lam_next[q], R.off[2 - j][2 - k], -i, X);
         }
-        f[q] = Storage<T>::kScaled ? v * float(weight<Q>(q)) : v;
-        // adjoint at t+1: from x + e_q (the mirrored pull)
-        if (kWalls && R.wall[2 - j][2 - k])
-            mu[q] = __ldg(g.lam_next[opposite<Q>(q)] + R.own + x);
-        else
-            mu[q] = __ldg(g.lam_next[q] + R.off[2 - j][2 - k] + xs[2 - i]);
-    }
-    const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
-    const long long c = dense_index(a.g, x, y, z);
-    float Fx, Fy, Fz;
-    cell_force(a, c, N, Fx, Fy, Fz);
-    const typename Rates<Q>::type r = load_rates<Q>(a);
-    float lam[Q], gx, gy, gz;
-    adjoint_collide<float>(f, Fx, Fy, Fz, r, mu, lam, gx, gy, gz);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) __stcs(g.lam_out[q] + R.own + x, lam[q]);
-    if (g.gF) {
-        g.gF[c] += gx;
-        g.gF[N + c] += gy;
-        g.gF[2 * N + c] += gz;
-    }
+    });
 }
 
-// The same adjoint step for two neighbouring cells (x0, x0 + 1) per thread in
-// packed f32x2 arithmetic (nx even).  The state is pulled as in step2_kernel;
-// the adjoint is pulled from the mirrored neighbours x + e_q: for e_x = 0 an
-// aligned pair, for e_x = +1 the cells (x0 + 1, x0 + 2), for e_x = -1
-// (x0 - 1, x0).
+// The adjoint step for two neighbouring cells (x0, x0 + 1) per thread in
+// packed f32x2 arithmetic.  The state is pulled as in step2_kernel; the adjoint
+// is pulled from the mirrored neighbours x + e_q: for e_x = 0 an aligned pair,
+// for e_x = +1 the cells (x0 + 1, x0 + 2), for e_x = -1 (x0 - 1, x0).
 // 3 blocks of 128 threads per SM: 168 registers.  D3Q27 spills a few of its
 // 242 there but beats 2 blocks and 4 (128 registers, ~700 B of spills:
 // 0.206 vs 0.135 ms at 128^3); D3Q15 fits without spills and beats 4 blocks
 // (276 B of spills; 0.098 vs 0.090 ms).
-template <int Q, typename T, bool kWalls>
+// kRag: ragged rows (PairCols).
+template <int Q, typename T, bool kWalls, bool kRag>
 __global__ void __launch_bounds__(128, 3) adjoint2_kernel(const StepIO<T> io, const AdjointArgs g,
                                                        const StepArgs a, const PackedRates pr) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-    const int x0 = 2 * t;
-    if (x0 >= a.g.nx || y >= a.g.ny) return;
+    if (2 * t >= row_end<float, kRag>(a.g.nx) || y >= a.g.ny) return;
+    const PairCols<kRag> X(2 * t, a.g.nx);
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
-    const int xm = (x0 == 0) ? a.g.nx - 1 : x0 - 1;
-    const int xp = (x0 + 2 == a.g.nx) ? 0 : x0 + 2;
-    const int own = R.own + x0;
     f2 f[Q], mu[Q];
-    static_for<Q>([&](auto iq) {
-        constexpr int q = decltype(iq)::value;
-        constexpr int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
-        constexpr int o = opposite<Q>(q);
-        f[q] = pull_pair<Q, T, kWalls>(io, R, q, x0, xm, xp);
-        if (kWalls && R.wall[2 - j][2 - k]) {
-            mu[q] = Pair<float>::ld2(g.lam_next[o] + own);
-        } else {
-            const float *row = g.lam_next[q] + R.off[2 - j][2 - k];
-            if constexpr (i == 0)
-                mu[q] = Pair<float>::ld2(row + x0);
-            else if constexpr (i == 1)
-                mu[q] = f2(__ldg(row + x0 + 1), __ldg(row + xp));
-            else
-                mu[q] = f2(__ldg(row + xm), __ldg(row + x0));
-        }
-    });
-    // deviations f - w: BF16 references added, 16-bit values scaled by w
-    if constexpr (Storage<T>::kRef) add_refs_pair<Q, kWalls>(io.ref_in, R, x0, xm, xp, f);
+    pull_pairs<Q, T>(io, R, X, f);
+    if (kWalls && (R.edge || blockDim.x < 32))
+        pull_adjoint<Q, kWalls>(g, R, X, mu);
+    else
+        pull_adjoint<Q, false>(g, R, X, mu);
+    even_lanes(X, mu);
+    // deviations f - w: 16-bit values scaled by w
     if constexpr (Storage<T>::kScaled) {
         static_for<Q>([&](auto iq) {
             constexpr int q = decltype(iq)::value;
@@ -149,42 +106,34 @@ __global__ void __launch_bounds__(128, 3) adjoint2_kernel(const StepIO<T> io, co
         });
     }
     const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
-    const long long c = dense_index(a.g, x0, y, z);
+    const long long c = dense_index(a.g, X.x0, y, z);
     f2 Fx, Fy, Fz;
-    if (a.Ffield) {  // 4-byte alignment only is required of the field: single loads
-        Fx = f2(__ldg(a.Ffield + c), __ldg(a.Ffield + c + 1));
-        Fy = f2(__ldg(a.Ffield + N + c), __ldg(a.Ffield + N + c + 1));
-        Fz = f2(__ldg(a.Ffield + 2 * N + c), __ldg(a.Ffield + 2 * N + c + 1));
-    } else {
-        Fx = f2(a.F[0]);
-        Fy = f2(a.F[1]);
-        Fz = f2(a.F[2]);
-    }
+    pair_force(a, X, y, z, Fx, Fy, Fz);
     // the dJ/dF accumulator is read now, so its latency hides behind the
     // collision's reverse; it is written back at the end
-    f2 a0 = f2(0.0f), a1 = f2(0.0f), a2 = f2(0.0f);
+    f2 acc[3] = {f2(0.0f), f2(0.0f), f2(0.0f)};
     if (g.gF) {
-        a0 = f2(g.gF[c], g.gF[c + 1]);
-        a1 = f2(g.gF[N + c], g.gF[N + c + 1]);
-        a2 = f2(g.gF[2 * N + c], g.gF[2 * N + c + 1]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float *p = g.gF + d * N + c;
+            acc[d] = f2(p[0], p[X.single() ? 0 : 1]);
+        }
     }
     const typename PairRates<Q>::type r = PairRates<Q>::load(pr);
-    f2 lam[Q], gx, gy, gz;
-    adjoint_collide<f2>(f, Fx, Fy, Fz, r, mu, lam, gx, gy, gz);
+    f2 lam[Q], gF[3];
+    adjoint_collide<f2>(f, Fx, Fy, Fz, r, mu, lam, gF[0], gF[1], gF[2]);
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
-        Pair<float>::st2(g.lam_out[q] + own, lam[q]);
+        Pair<float>::st2(element<kRag>(g.lam_out[q], R.own + X.at), lam[q]);
     });
-    if (g.gF) {
-        a0 = a0 + gx;
-        a1 = a1 + gy;
-        a2 = a2 + gz;
-        g.gF[c] = a0.lo();
-        g.gF[c + 1] = a0.hi();
-        g.gF[N + c] = a1.lo();
-        g.gF[N + c + 1] = a1.hi();
-        g.gF[2 * N + c] = a2.lo();
-        g.gF[2 * N + c + 1] = a2.hi();
+    if (g.gF && (!kRag || X.at == X.x0)) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            float *p = g.gF + d * N + c;
+            acc[d] = acc[d] + gF[d];
+            p[0] = acc[d].lo();
+            if (!X.single()) p[1] = acc[d].hi();
+        }
     }
 }
 
@@ -283,32 +232,21 @@ __global__ void __launch_bounds__(128, 8) energy_kernel(const StepIO<T> io, cons
 template <int Q, typename T>
 cudaError_t launch_adjoint(const void *f_t, const float *lam_next, float *lam_out, float *gF,
                            const StepArgs &a, cudaStream_t st) {
-    StepIO<T> io{};  // slots q >= Q stay null
+    const StepIO<T> io = step_io<Q, T>(f_t, nullptr, a.g);
     AdjointArgs g{};
     for (int q = 0; q < Q; ++q) {
-        io.in[q] = static_cast<const T *>(f_t) + q * a.g.pop;
-        io.out[q] = nullptr;
         g.lam_next[q] = lam_next + q * a.g.pop;
         g.lam_out[q] = lam_out + q * a.g.pop;
     }
-    io.ref_in = Storage<T>::kRef ? ref_array<Q>(static_cast<const T *>(f_t), a.g.pop, 0) : nullptr;
     g.gF = gF;
-    if (a.g.nx % 2 == 0) {
-        Grid half = a.g;
-        half.nx = a.g.nx / 2;
-        const CellLaunch L = cell_launch(half);
-        const PackedRates pr = packed_rates(a);
-        if (a.g.bc)
-            adjoint2_kernel<Q, T, true><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
-        else
-            adjoint2_kernel<Q, T, false><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
-        return cudaGetLastError();
-    }
-    const CellLaunch L = cell_launch(a.g);
-    if (a.g.bc)
-        adjoint_kernel<Q, T, true><<<L.grid, L.block, 0, st>>>(io, g, a);
+    const CellLaunch L = pair_launch(a.g, stored_row<float>(a.g.nx));
+    const PackedRates pr = packed_rates(a);
+    if (ragged<float>(a.g))  // one instantiation, with the wall selects: the rarer case
+        adjoint2_kernel<Q, T, true, true><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
+    else if (a.g.bc)
+        adjoint2_kernel<Q, T, true, false><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
     else
-        adjoint_kernel<Q, T, false><<<L.grid, L.block, 0, st>>>(io, g, a);
+        adjoint2_kernel<Q, T, false, false><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
     return cudaGetLastError();
 }
 

@@ -93,38 +93,6 @@ __device__ __forceinline__ Rates15<float> load_rates<15>(const StepArgs &a) {
     return r;
 }
 
-template <int Q>
-__device__ __forceinline__ void collide(float (&f)[Q], float Fx, float Fy, float Fz,
-                                        const typename Rates<Q>::type &r, bool has_force);
-template <>
-__device__ __forceinline__ void collide<27>(float (&f)[27], float Fx, float Fy, float Fz,
-                                            const Rates27<float> &r, bool) {
-    collide27<float>(f, Fx, Fy, Fz, r);
-}
-template <>
-__device__ __forceinline__ void collide<15>(float (&f)[15], float Fx, float Fy, float Fz,
-                                            const Rates15<float> &r, bool has_force) {
-    collide15<float>(f, Fx, Fy, Fz, r, has_force);
-}
-
-// The same, returning the cell's velocity (Eq. velocitycalculation).
-template <int Q>
-__device__ __forceinline__ void collide_u(float (&f)[Q], float Fx, float Fy, float Fz,
-                                          const typename Rates<Q>::type &r, bool has_force,
-                                          float &ux, float &uy, float &uz);
-template <>
-__device__ __forceinline__ void collide_u<27>(float (&f)[27], float Fx, float Fy, float Fz,
-                                              const Rates27<float> &r, bool, float &ux, float &uy,
-                                              float &uz) {
-    collide27<float>(f, Fx, Fy, Fz, r, ux, uy, uz);
-}
-template <>
-__device__ __forceinline__ void collide_u<15>(float (&f)[15], float Fx, float Fy, float Fz,
-                                              const Rates15<float> &r, bool has_force, float &ux,
-                                              float &uy, float &uz) {
-    collide15<float>(f, Fx, Fy, Fz, r, has_force, ux, uy, uz);
-}
-
 // The change d = f~ - f the collision makes (for the incremental update).
 template <int Q>
 __device__ __forceinline__ void collide_delta(const float (&f)[Q], float Fx, float Fy, float Fz,
@@ -182,6 +150,24 @@ struct StepIO {
     float4 *ref_out;       // and of the output state
 };
 
+// Element e of a plane.  The offset is an unsigned 32-bit number of bytes, which
+// the hardware adds to a uniform base in the access itself, where a signed
+// element offset costs a 64-bit multiply-add per access on the FMA pipe (us a
+// step: D3Q15 256^3 FP16 210 -> 201, BF16 229 -> 220; D3Q27 FP32 64^3 6.92 -> 6.76,
+// 80^3 19.8 -> 18.6).  Planes of more than 2^32 bytes (FP32, over 2^30 elements) take
+// the instantiations for ragged rows, which keep element offsets for FP32.
+// kPlain: element offsets whatever the type, where those measured faster: the
+// 16-bit D3Q27 step (256^3: FP16 327 against 338 us, BF16 391 against 398), whose
+// registers are short, and some in-place kernels (kAAPlain).
+template <bool kRag, bool kPlain = false, typename T>
+__device__ __forceinline__ T *element(T *plane, int e) {
+    using Byte = typename std::conditional<std::is_const<T>::value, const char, char>::type;
+    if constexpr (kPlain || (kRag && sizeof(T) == 4))
+        return plane + e;
+    else
+        return reinterpret_cast<T *>(reinterpret_cast<Byte *>(plane) +
+                                     unsigned(e) * unsigned(sizeof(T)));
+}
 // 2-cell pair helpers for the packed kernel (x0 even, row pitch even).
 template <typename T>
 struct Pair;
@@ -326,6 +312,7 @@ template <bool kWalls>
 struct Rows {
     int off[3][3];
     bool wall[3][3];
+    bool edge;  // some source is beyond a wall: the others take the plain loads
     int own;
 };
 
@@ -348,8 +335,55 @@ __device__ __forceinline__ Rows<kWalls> pull_rows(const Grid &g, int y, int z) {
             r.off[j][k] = (zs[k] * g.ny + ys[j]) * g.px;
             r.wall[j][k] = kWalls && (wy[j] || wz[k]);
         }
+    r.edge = wy[0] || wy[2] || wz[0] || wz[2];
     r.own = (z * g.ny + y) * g.px;
     return r;
+}
+
+// Cells a row's stores cover: the row rounded up to whole 32-byte sectors (the
+// pitch has room).  A sector that is stored in part has to be filled from DRAM:
+// D3Q27 FP32 at 126 x 117 x 133 cells took 76.2 us a step, at 128 (no partial
+// sector) 64.9 us.  The threads past the row's end repeat its last cells and
+// store them there, in the same instructions as the rest of their warp.
+template <typename T>
+__host__ __device__ constexpr int stored_row(int nx) {
+    constexpr int n = 32 / int(sizeof(T));
+    return (nx + n - 1) / n * n;
+}
+
+// Columns of a thread's two cells (x0, x0 + 1), x0 even, and of their sources:
+// xm left of x0, x1 (= x0 + 1 inside the row) right of x0, xp right of x0 + 1;
+// at: where the thread stores.
+// kRag: rows that do not fill their last sector.  The threads past the end
+// (at >= nx) repeat the last pair.  In a row of odd length the last pair is one
+// cell: its high lane reads in-range elements, is set to the low lane once the
+// values are in registers (even_lanes) and stored in the row's padding.
+template <bool kRag>
+struct PairCols {
+    int at, x0, xm, xp, nx;
+    __device__ __forceinline__ PairCols(int x, int n) : at(x), x0(x), nx(n) {
+        if (kRag) x0 = min(x0, (nx - 1) & ~1);
+        xm = (x0 == 0) ? nx - 1 : x0 - 1;
+        xp = (kRag ? x0 + 2 >= nx : x0 + 2 == nx) ? 0 : x0 + 2;
+    }
+    __device__ __forceinline__ bool single() const { return kRag && x0 + 1 == nx; }
+    __device__ __forceinline__ int x1() const { return single() ? 0 : x0 + 1; }
+};
+
+// End of the cells a row's threads store (T: the type stored).
+template <typename T, bool kRag>
+__device__ __forceinline__ int row_end(int nx) {
+    return kRag ? stored_row<T>(nx) : nx;
+}
+
+template <int Q, bool kRag>
+__device__ __forceinline__ void even_lanes(const PairCols<kRag> &X, f2 (&f)[Q]) {
+    if constexpr (kRag) {
+        if (X.single()) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) f[q] = f2(f[q].lo(), f[q].lo());
+        }
+    }
 }
 
 // BF16 momentum references (see lattice.cuh) for the pair kernels.
@@ -379,28 +413,29 @@ __device__ __forceinline__ float4 load_ref(const float4 *p) {
     }
 }
 
-template <int Q, bool kWalls>
+// kSel: with the wall selects.
+template <int Q, bool kSel, bool kWalls, bool kRag>
 __device__ __forceinline__ void add_refs_pair(const float4 *__restrict__ ref, const Rows<kWalls> &R,
-                                              int x0, int xm, int xp, f2 (&f)[Q]) {
+                                              const PairCols<kRag> &X, f2 (&f)[Q]) {
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         if constexpr (has_ref<Q>(q)) {
             constexpr int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
             constexpr int cy = ey<Q>(q), cz = ez<Q>(q);
             float rlo, rhi;
-            if (kWalls && R.wall[j][k]) {
-                rlo = rhi = -ref_dot<Q, q>(load_ref<cy, cz>(ref + ((R.own + x0) >> 1)));
+            if (kSel && R.wall[j][k]) {
+                rlo = rhi = -ref_dot<Q, q>(load_ref<cy, cz>(ref + ((R.own + X.x0) >> 1)));
             } else {
                 const float4 *row = ref + (R.off[j][k] >> 1);
-                const float4 C = load_ref<cy, cz>(row + (x0 >> 1));
+                const float4 C = load_ref<cy, cz>(row + (X.x0 >> 1));
                 if constexpr (i == 0) {
                     rlo = rhi = ref_dot<Q, q>(C);
                 } else if constexpr (i == 1) {
-                    rlo = ref_dot<Q, q>(load_ref<cy, cz>(row + (xm >> 1)));
+                    rlo = ref_dot<Q, q>(load_ref<cy, cz>(row + (X.xm >> 1)));
                     rhi = ref_dot<Q, q>(C);
                 } else {
-                    rlo = ref_dot<Q, q>(C);
-                    rhi = ref_dot<Q, q>(load_ref<cy, cz>(row + (xp >> 1)));
+                    rlo = ref_dot<Q, q>(kRag ? load_ref<cy, cz>(row + (X.x1() >> 1)) : C);
+                    rhi = ref_dot<Q, q>(load_ref<cy, cz>(row + (X.xp >> 1)));
                 }
             }
             f[q] = f[q] + f2(rlo, rhi);
@@ -590,80 +625,153 @@ __device__ __forceinline__ float deviation(double f) {
     return float(f - w);
 }
 
-// One fused step, one cell per thread: pull-gather (streaming with
-// bounce-back), collision, store.  With BF16 momentum references the cells
-// x (even) and x + 1, held by neighbouring lanes, exchange their velocities
-// for the pair's reference, so every lane takes part: cells beyond the grid
-// edge compute on a clamped cell and store nothing.
-// kSR (FP32 storage, opt-in): the update is f~ = f + d with d the
-// collision's change, and that last addition is rounded stochastically
-// (add_sr32), so that no rounding error repeats identically step after step
-// at a steady state.
-template <int Q, typename T, bool kWalls, bool kSR = false>
-__global__ void __launch_bounds__(128) step_kernel(const StepIO<T> io, const StepArgs a) {
-    int x, y, z;
-    const bool inside = cell_coords(a.g, x, y, z);
-    if constexpr (Storage<T>::kRef) {
-        x = min(x, a.g.nx - 1);
-        y = min(y, a.g.ny - 1);
-    } else {
-        if (!inside) return;
-    }
-    const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
-    const int xs[3] = {(x + 1 == a.g.nx) ? 0 : x + 1, x, (x == 0) ? a.g.nx - 1 : x - 1};
-    float f[Q];
+// One cell's pulled FP32 populations.
+// kRag: see element().
+template <int Q, bool kRag, bool kWalls>
+__device__ __forceinline__ void pull_cell(const StepIO<float> &io, const Rows<kWalls> &R, int x,
+                                          int nx, float (&f)[Q]) {
+    const int xs[3] = {(x + 1 == nx) ? 0 : x + 1, x, (x == 0) ? nx - 1 : x - 1};
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         constexpr int i = ex<Q>(q) + 1, j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
         const bool wall = kWalls && R.wall[j][k];
         const int src = wall ? R.own + x : R.off[j][k] + xs[i];
-        const T *plane = wall ? io.in[opposite<Q>(q)] : io.in[q];
-        float v = Storage<T>::load(plane + src);
-        if constexpr (Storage<T>::kRef && has_ref<Q>(q)) {
-            const float r = ref_dot<Q, q>(__ldg(io.ref_in + (src >> 1)));
-            v += wall ? -r : r;
-        }
-        f[q] = Storage<T>::kScaled ? v * float(weight<Q>(q)) : v;
+        f[q] = Pair<float>::ld1(element<kRag>(wall ? io.in[opposite<Q>(q)] : io.in[q], src));
     });
+}
+
+// One fused FP32 step, one cell per thread, for small grids with rows of odd
+// length.  A small grid does not fill the chip and its step takes as long as
+// one thread's chain of instructions, which is shorter here.  (Scalar
+// arithmetic rounds differently from the packed one, so grids that can also run
+// in place, with even rows, keep the two-cell kernel at every size: their
+// states are the same bit for bit in either scheme.)  See kSmallCells.
+template <int Q, bool kWalls, bool kForm>
+__global__ void __launch_bounds__(128) step1_kernel(const StepIO<float> io, const StepArgs a) {
+    int x, y, z;
+    if (!cell_coords(a.g, x, y, z)) return;
+    const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
+    float f[Q];
+    pull_cell<Q, false>(io, R, x, a.g.nx, f);
+    const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
+    float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f, ux, uy, uz;
+    if (Q == 27 || kForm) cell_force(a, dense_index(a.g, x, y, z), N, Fx, Fy, Fz);
+    const typename Rates<Q>::type r = load_rates<Q>(a);
+    if constexpr (Q == 27)
+        // periodic, the general form schedules better (9^3: 2.20 / 2.39 us; walled
+        // 2.65 / 2.27)
+        collide27_g<float, false, kForm && kWalls>(f, Fx, Fy, Fz, r, ux, uy, uz);
+    else
+        collide15<float>(f, Fx, Fy, Fz, r, kForm, ux, uy, uz);
+    static_for<Q>([&](auto iq) {
+        constexpr int q = decltype(iq)::value;
+        __stcs(element<false>(io.out[q], R.own + x), f[q] * store_scale<Q, float>(q));
+    });
+}
+
+// One fused step with the stochastically rounded FP32 update (LBM_F32_SR), one
+// cell per thread: the update is f~ = f + d with d the collision's change, and
+// that last addition is rounded stochastically (add_sr32), so that no rounding
+// error repeats identically step after step at a steady state.
+template <int Q, bool kWalls>
+__global__ void __launch_bounds__(128) step_sr32_kernel(const StepIO<float> io, const StepArgs a) {
+    int x, y, z;
+    if (!cell_coords(a.g, x, y, z)) return;
+    const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
+    float f[Q];
+    pull_cell<Q, true>(io, R, x, a.g.nx, f);
     const unsigned seed = cell_seed<Q>(f, R.own + x);
     float Fx, Fy, Fz;
     const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
     cell_force(a, dense_index(a.g, x, y, z), N, Fx, Fy, Fz);
     const typename Rates<Q>::type r = load_rates<Q>(a);
-    float ux, uy, uz;
-    if constexpr (kSR) {
-        float d[Q];
-        collide_delta<Q>(f, Fx, Fy, Fz, r, a.has_force != 0, d);
-        static_for<Q>([&](auto iq) {
-            constexpr int q = decltype(iq)::value;
-            f[q] = add_sr32(f[q], d[q], sr_bits<q>(seed));
-        });
-    } else {
-        collide_u<Q>(f, Fx, Fy, Fz, r, a.has_force != 0, ux, uy, uz);
-    }
-    float4 J = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if constexpr (Storage<T>::kRef) {
-        const float px = __shfl_xor_sync(0xffffffffu, ux, 1);
-        const float py = __shfl_xor_sync(0xffffffffu, uy, 1);
-        const float pz = __shfl_xor_sync(0xffffffffu, uz, 1);
-        if ((x ^ 1) < a.g.nx)  // both cells of the pair exist (a + b == b + a exactly)
-            J = make_float4(1.5f * (ux + px), 1.5f * (uy + py), 1.5f * (uz + pz), 0.0f);
-        else
-            J = make_float4(3.0f * ux, 3.0f * uy, 3.0f * uz, 0.0f);
-        J.w = J.x;
-        if (!inside) return;
-        if ((x & 1) == 0) __stcs(io.ref_out + ((R.own + x) >> 1), J);
-    }
+    float d[Q];
+    collide_delta<Q>(f, Fx, Fy, Fz, r, a.has_force != 0, d);
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
-        float ref = 0.0f;
-        if constexpr (Storage<T>::kRef && has_ref<Q>(q)) ref = ref_dot<Q, q>(J);
-        store_dev_step<Q, T, q>(io.out[q] + R.own + x, f[q], seed, ref);
+        __stcs(io.out[q] + (R.own + x), add_sr32(f[q], d[q], sr_bits<q>(seed)));
     });
 }
 
+// The values of a plane's row (offset of its start) at x0 - i and x0 + 1 - i.
+// kRowFirst: the row's pointer, then the column (see kAAPlain).
+template <bool kPlain = false, bool kRowFirst = false, typename T, bool kRag>
+__device__ __forceinline__ f2 ld_shifted(const T *plane, int row, int i, const PairCols<kRag> &X) {
+    if constexpr (kRowFirst) {
+        plane += row;
+        row = 0;
+    }
+    const T *own = element<kRag, kPlain>(plane, row + X.x0);
+    if (i == 0) return Pair<T>::ld2(own);
+    if (i == 1)
+        return f2(Pair<T>::ld1(element<kRag, kPlain>(plane, row + X.xm)), Pair<T>::ld1(own));
+    return f2(Pair<T>::ld1(kRag ? element<kRag, kPlain>(plane, row + X.x1()) : own + 1),
+              Pair<T>::ld1(element<kRag, kPlain>(plane, row + X.xp)));
+}
+
+// Pair gather: population q of cells (x0, x0 + 1) from the pull sources.
+template <int Q, typename T>
+constexpr bool kStepPlain = Q == 27 && Storage<T>::kScaled;
+
+template <int Q, typename T, bool kSel, bool kWalls, bool kRag>
+__device__ __forceinline__ f2 pull_pair(const StepIO<T> &io, const Rows<kWalls> &R, int q,
+                                        const PairCols<kRag> &X) {
+    const int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
+    if (kSel && R.wall[j][k])
+        return Pair<T>::ld2(
+            element<kRag, kStepPlain<Q, T>>(io.in[opposite<Q>(q)], R.own + X.x0));
+    return ld_shifted<kStepPlain<Q, T>>(io.in[q], R.off[j][k], i, X);
+}
+
+// All populations of the pair as stored, BF16 references added.  The wall
+// selects are compiled beside the plain loads and taken by the rows along a
+// wall only: with selects everywhere the 128 x 117 x 133 step took 69.5 us
+// between walls against 64.9 us periodic.
+// kShort: rows of less than a warp, where one warp holds rows of both kinds and
+// would run both: the selects alone.
+template <int Q, typename T, bool kShort = false, bool kWalls, bool kRag>
+__device__ __forceinline__ void pull_pairs(const StepIO<T> &io, const Rows<kWalls> &R,
+                                           const PairCols<kRag> &X, f2 (&f)[Q]) {
+    const auto pull = [&](auto sel) {
+        constexpr bool kSel = decltype(sel)::value;
+        static_for<Q>([&](auto iq) {
+            constexpr int q = decltype(iq)::value;
+            f[q] = pull_pair<Q, T, kSel>(io, R, q, X);
+        });
+        if constexpr (Storage<T>::kRef) add_refs_pair<Q, kSel>(io.ref_in, R, X, f);
+    };
+    if constexpr (kShort) {
+        pull(std::integral_constant<bool, kWalls>{});
+    } else {
+        if (kWalls && (R.edge || blockDim.x < 32))
+            pull(std::integral_constant<bool, kWalls>{});
+        else
+            pull(std::false_type{});
+    }
+    even_lanes(X, f);
+}
+
+// Body force of the pair (x0, x0 + 1): the field (4-byte alignment only is
+// required of it: single loads), else the uniform force.
+template <bool kRag = false>
+__device__ __forceinline__ void pair_force(const StepArgs &a, const PairCols<kRag> &X, int y, int z,
+                                           f2 &Fx, f2 &Fy, f2 &Fz) {
+    if (a.Ffield) {
+        const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
+        const float *p = a.Ffield + dense_index(a.g, X.x0, y, z);
+        const int n = X.single() ? 0 : 1;
+        Fx = f2(__ldg(p), __ldg(p + n));
+        Fy = f2(__ldg(p + N), __ldg(p + N + n));
+        Fz = f2(__ldg(p + 2 * N), __ldg(p + 2 * N + n));
+    } else {
+        Fx = f2(a.F[0]);
+        Fy = f2(a.F[1]);
+        Fz = f2(a.F[2]);
+    }
+}
+
 // One fused D3Q27 step, two neighbouring cells (x0, x0 + 1) per thread with
-// the collision in packed f32x2 arithmetic.  nx must be even.  Loads of
+// the collision in packed f32x2 arithmetic.  Loads of
 // populations with e_x = 0 and all stores are aligned 2-element accesses;
 // e_x = +-1 sources are two single loads (x0 - 1, x0) or (x0 + 1, x0 + 2).
 // Blocks of 128 per SM, by measurement: FP32 storage 5 (96 registers, no
@@ -675,95 +783,40 @@ template <typename T>
 constexpr int kStep2Blocks = Storage<T>::kScaled ? 6 : 5;
 
 // kEq: the rates from the trace on are all 1 (relax27).
-template <typename T, bool kWalls, bool kEq>
+// kShort: see pull_pairs.
+template <typename T, bool kWalls, bool kEq, bool kRag, bool kShort = false>
 __global__ void __launch_bounds__(128, kStep2Blocks<T>) step2_kernel(const StepIO<T> io,
                                                                   const StepArgs a,
                                                                   const PackedRates pr) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-    const int x0 = 2 * t;
-    if (x0 >= a.g.nx || y >= a.g.ny) return;
+    if (2 * t >= row_end<T, kRag>(a.g.nx) || y >= a.g.ny) return;
+    const PairCols<kRag> X(2 * t, a.g.nx);
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
-    const int xm = (x0 == 0) ? a.g.nx - 1 : x0 - 1;
-    const int xp = (x0 + 2 == a.g.nx) ? 0 : x0 + 2;
-    f2 f[27];
-#pragma unroll
-    for (int q = 0; q < 27; ++q) {
-        const int i = ex<27>(q), j = ey<27>(q) + 1, k = ez<27>(q) + 1;
-        f2 v;
-        if (kWalls && R.wall[j][k]) {
-            v = Pair<T>::ld2(io.in[opposite<27>(q)] + R.own + x0);
-        } else {
-            const T *row = io.in[q] + R.off[j][k];
-            if (i == 0)
-                v = Pair<T>::ld2(row + x0);
-            else if (i == 1)
-                v = f2(Pair<T>::ld1(row + xm), Pair<T>::ld1(row + x0));
-            else
-                v = f2(Pair<T>::ld1(row + x0 + 1), Pair<T>::ld1(row + xp));
-        }
-        f[q] = v;  // weight-scaled 16-bit values go in as stored (collide27_g)
-    }
-    if constexpr (Storage<T>::kRef) add_refs_pair<27, kWalls>(io.ref_in, R, x0, xm, xp, f);
-    const unsigned seed = pair_seed<27>(f, R.own + x0);
+    f2 f[27];  // weight-scaled 16-bit values go in as stored (collide27_g)
+    pull_pairs<27, T, kShort>(io, R, X, f);
+    const int own = R.own + X.x0;
+    const unsigned seed = pair_seed<27>(f, own);
     f2 Fx, Fy, Fz;
-    if (a.Ffield) {
-        const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
-        const long long c = dense_index(a.g, x0, y, z);
-        Fx = f2(__ldg(a.Ffield + c), __ldg(a.Ffield + c + 1));
-        Fy = f2(__ldg(a.Ffield + N + c), __ldg(a.Ffield + N + c + 1));
-        Fz = f2(__ldg(a.Ffield + 2 * N + c), __ldg(a.Ffield + 2 * N + c + 1));
-    } else {
-        Fx = f2(a.F[0]);
-        Fy = f2(a.F[1]);
-        Fz = f2(a.F[2]);
-    }
+    pair_force(a, X, y, z, Fx, Fy, Fz);
     const Rates27<f2> r = load_rates_packed(pr);
     f2 ux, uy, uz;
     collide27_g<f2, Storage<T>::kScaled, kEq>(f, Fx, Fy, Fz, r, ux, uy, uz);
     float4 J = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if constexpr (Storage<T>::kRef) {
         J = pair_ref(ux, uy, uz);
-        __stcs(io.ref_out + ((R.own + x0) >> 1), J);
+        __stcs(io.ref_out + ((R.own + X.at) >> 1), J);
     }
     static_for<27>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         const f2 v = stored_pair<27, T, q>(f[q], store_scale<27, T>(q), J);
-        Pair<T>::template st2s<q>(io.out[q] + R.own + x0, v, seed);
+        Pair<T>::template st2s<q>(element<kRag, kStepPlain<27, T>>(io.out[q], R.own + X.at), v,
+                                  seed);
     });
 }
 
-// Pair gather for lattice Q: population q of cells (x0, x0 + 1) from the pull
-// sources (see step2_kernel).
-template <int Q, typename T, bool kWalls>
-__device__ __forceinline__ f2 pull_pair(const StepIO<T> &io, const Rows<kWalls> &R, int q, int x0,
-                                        int xm, int xp) {
-    const int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
-    if (kWalls && R.wall[j][k]) return Pair<T>::ld2(io.in[opposite<Q>(q)] + R.own + x0);
-    const T *row = io.in[q] + R.off[j][k];
-    if (i == 0) return Pair<T>::ld2(row + x0);
-    if (i == 1) return f2(Pair<T>::ld1(row + xm), Pair<T>::ld1(row + x0));
-    return f2(Pair<T>::ld1(row + x0 + 1), Pair<T>::ld1(row + xp));
-}
-
-// Body force of the pair (x0, x0 + 1): the field, else the uniform force.
-__device__ __forceinline__ void pair_force(const StepArgs &a, int x0, int y, int z, f2 &Fx, f2 &Fy,
-                                           f2 &Fz) {
-    if (a.Ffield) {
-        const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
-        const long long c = dense_index(a.g, x0, y, z);
-        Fx = f2(__ldg(a.Ffield + c), __ldg(a.Ffield + c + 1));
-        Fy = f2(__ldg(a.Ffield + N + c), __ldg(a.Ffield + N + c + 1));
-        Fz = f2(__ldg(a.Ffield + 2 * N + c), __ldg(a.Ffield + 2 * N + c + 1));
-    } else {
-        Fx = f2(a.F[0]);
-        Fy = f2(a.F[1]);
-        Fz = f2(a.F[2]);
-    }
-}
-
 // One fused D3Q15 step, two neighbouring cells per thread in packed f32x2
-// arithmetic (nx even); loads and stores as in step2_kernel.
+// arithmetic; loads and stores as in step2_kernel.
 // kForce = false (no force anywhere) compiles the force-free cascade alone:
 // without the forced path beside it the kernel needs fewer registers (no
 // spills at 5 blocks per SM with 16-bit storage, against 104-128 bytes;
@@ -774,22 +827,17 @@ __device__ __forceinline__ void pair_force(const StepArgs &a, int x0, int y, int
 template <typename T, bool kForce>
 constexpr int kQ15Blocks = Storage<T>::kScaled ? (kForce ? 5 : 6) : 4;
 
-template <typename T, bool kWalls, bool kForce>
+template <typename T, bool kWalls, bool kForce, bool kRag, bool kShort = false>
 __global__ void __launch_bounds__(128, (kQ15Blocks<T, kForce>))
     step2_q15_kernel(const StepIO<T> io, const StepArgs a, const PackedRates pr) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-    const int x0 = 2 * t;
-    if (x0 >= a.g.nx || y >= a.g.ny) return;
+    if (2 * t >= row_end<T, kRag>(a.g.nx) || y >= a.g.ny) return;
+    const PairCols<kRag> X(2 * t, a.g.nx);
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
-    const int xm = (x0 == 0) ? a.g.nx - 1 : x0 - 1;
-    const int xp = (x0 + 2 == a.g.nx) ? 0 : x0 + 2;
+    const int own = R.own + X.x0;
     f2 f[15];
-    static_for<15>([&](auto iq) {
-        constexpr int q = decltype(iq)::value;
-        f[q] = pull_pair<15, T, kWalls>(io, R, q, x0, xm, xp);
-    });
-    if constexpr (Storage<T>::kRef) add_refs_pair<15, kWalls>(io.ref_in, R, x0, xm, xp, f);
+    pull_pairs<15, T, kShort>(io, R, X, f);
     if constexpr (Storage<T>::kScaled) {
         static_for<15>([&](auto iq) {
             constexpr int q = decltype(iq)::value;
@@ -797,9 +845,9 @@ __global__ void __launch_bounds__(128, (kQ15Blocks<T, kForce>))
         });
     }
     unsigned seed = 0;
-    if constexpr (!kSeedAfterCollision<15, T>) seed = pair_seed<15>(f, R.own + x0);
+    if constexpr (!kSeedAfterCollision<15, T>) seed = pair_seed<15>(f, own);
     f2 Fx = f2(0.0f), Fy = f2(0.0f), Fz = f2(0.0f);
-    if constexpr (kForce) pair_force(a, x0, y, z, Fx, Fy, Fz);
+    if constexpr (kForce) pair_force(a, X, y, z, Fx, Fy, Fz);
     Rates15<f2> r;
 #pragma unroll
     for (int b = 0; b < 15; ++b) r.w[b] = f2(pr.w15[b]);
@@ -808,13 +856,14 @@ __global__ void __launch_bounds__(128, (kQ15Blocks<T, kForce>))
     float4 J = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if constexpr (Storage<T>::kRef) {
         J = pair_ref(ux, uy, uz);
-        __stcs(io.ref_out + ((R.own + x0) >> 1), J);
+        __stcs(io.ref_out + ((R.own + X.at) >> 1), J);
     }
-    if constexpr (kSeedAfterCollision<15, T>) seed = pair_seed<15>(f, R.own + x0);
+    if constexpr (kSeedAfterCollision<15, T>) seed = pair_seed<15>(f, own);
     static_for<15>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         const f2 v = stored_pair<15, T, q>(f[q], store_scale<15, T>(q), J);
-        Pair<T>::template st2s<q>(io.out[q] + R.own + x0, v, seed);
+        Pair<T>::template st2s<q>(element<kRag, kStepPlain<15, T>>(io.out[q], R.own + X.at), v,
+                                  seed);
     });
 }
 
@@ -857,10 +906,10 @@ struct PairCollide<15> {
 
 // Raw pulled values -> the collision's inputs: BF16 references added (their
 // producers are the pull sources, see lattice.cuh), then the load scale.
-template <int Q, typename T, bool kWalls>
-__device__ __forceinline__ void pair_inputs(const StepIO<T> &io, const Rows<kWalls> &R, int x0,
-                                            int xm, int xp, f2 (&f)[Q]) {
-    if constexpr (Storage<T>::kRef) add_refs_pair<Q, kWalls>(io.ref_in, R, x0, xm, xp, f);
+template <int Q, typename T, bool kWalls, bool kRag>
+__device__ __forceinline__ void pair_inputs(const StepIO<T> &io, const Rows<kWalls> &R,
+                                            const PairCols<kRag> &X, f2 (&f)[Q]) {
+    if constexpr (Storage<T>::kRef) add_refs_pair<Q, kWalls>(io.ref_in, R, X, f);
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         constexpr float sc = load_scale<Q, T>(q);
@@ -869,12 +918,13 @@ __device__ __forceinline__ void pair_inputs(const StepIO<T> &io, const Rows<kWal
 }
 
 // The collision of an in-place step, then the pair's reference (BF16).
-template <int Q, typename T, bool kEq, bool kForce>
+template <int Q, typename T, bool kEq, bool kForce, bool kRag>
 __device__ __forceinline__ float4 pair_collide(const StepIO<T> &io, const StepArgs &a,
-                                               const PackedRates &pr, int x0, int y, int z,
-                                               int own, f2 (&f)[Q]) {
+                                               const PackedRates &pr,
+                                               const PairCols<kRag> &X, int y, int z, int own,
+                                               f2 (&f)[Q]) {
     f2 Fx = f2(0.0f), Fy = f2(0.0f), Fz = f2(0.0f), ux, uy, uz;
-    if constexpr (kForce) pair_force(a, x0, y, z, Fx, Fy, Fz);
+    if constexpr (kForce) pair_force(a, X, y, z, Fx, Fy, Fz);
     PairCollide<Q>::template run<kFoldedLoad<Q, T>(), kEq, kForce>(f, Fx, Fy, Fz, pr, ux, uy, uz);
     float4 J = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if constexpr (Storage<T>::kRef) {
@@ -884,31 +934,40 @@ __device__ __forceinline__ float4 pair_collide(const StepIO<T> &io, const StepAr
     return J;
 }
 
-template <int Q, typename T, bool kWalls, bool kEq, bool kForce>
+// Element offsets instead of byte offsets (element()) where those measured slower
+// in the in-place kernels: 256^3 us a step, bytes / elements, D3Q27 BF16 466 / 411
+// (452 with row and column summed first), FP32 at general rates 545 / 527 (598);
+// ragged rows (250 x 256 x 256, a wall) FP16 511 / 356 (407 row first); else
+// bytes: D3Q27 FP16 321 / 353, D3Q15 FP16 203 / 231.
+template <int Q, typename T, bool kEq, bool kRag>
+constexpr bool kAAPlain = kRag || (Q == 27 && (Storage<T>::kRef || (sizeof(T) == 4 && !kEq)));
+
+template <int Q, typename T, bool kWalls, bool kEq, bool kForce, bool kRag>
 __global__ void __launch_bounds__(128) aa_even_kernel(const StepIO<T> io, const StepArgs a,
                                                       const PackedRates pr) {
+    constexpr bool kPlain = kAAPlain<Q, T, kEq, kRag>;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-    const int x0 = 2 * t;
-    if (x0 >= a.g.nx || y >= a.g.ny) return;
+    if (2 * t >= row_end<T, kRag>(a.g.nx) || y >= a.g.ny) return;
+    const PairCols<kRag> X(2 * t, a.g.nx);
+    const int x0 = X.x0;
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);  // producers of the values (BF16)
-    const int xm = (x0 == 0) ? a.g.nx - 1 : x0 - 1;
-    const int xp = (x0 + 2 == a.g.nx) ? 0 : x0 + 2;
     const int own = R.own + x0;
     f2 f[Q];
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
-        f[q] = Pair<T>::ld2(io.in[q] + own);
+        f[q] = Pair<T>::ld2(element<kRag, kPlain>(io.in[q], own));
     });
-    pair_inputs<Q, T, kWalls>(io, R, x0, xm, xp, f);
+    pair_inputs<Q, T>(io, R, X, f);
     unsigned seed = 0;
     if constexpr (!kSeedAfterCollision<Q, T>) seed = pair_seed<Q>(f, own);
-    const float4 J = pair_collide<Q, T, kEq, kForce>(io, a, pr, x0, y, z, own, f);
+    const float4 J = pair_collide<Q, T, kEq, kForce>(io, a, pr, X, y, z, own, f);
     if constexpr (kSeedAfterCollision<Q, T>) seed = pair_seed<Q>(f, own);
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         const f2 v = stored_pair<Q, T, q>(f[q], store_scale<Q, T>(q), J);
-        Pair<T>::template st2s<q>(io.out[opposite<Q>(q)] + own, v, seed);
+        Pair<T>::template st2s<q>(element<kRag, kPlain>(io.out[opposite<Q>(q)], R.own + X.at), v,
+                                  seed);
     });
 }
 
@@ -919,59 +978,69 @@ __global__ void __launch_bounds__(128) aa_even_kernel(const StepIO<T> io, const 
 template <int Q, typename T, bool kForce>
 constexpr int kAAOddBlocks = Q == 27 ? 5 : (kForce ? 4 : 5);
 
-template <int Q, typename T, bool kWalls, bool kEq, bool kForce>
+template <int Q, typename T, bool kWalls, bool kEq, bool kForce, bool kRag>
 __global__ void __launch_bounds__(128, (kAAOddBlocks<Q, T, kForce>))
     aa_odd_kernel(const StepIO<T> io, const StepArgs a, const PackedRates pr) {
+    constexpr bool kPlain = kAAPlain<Q, T, kEq, kRag>;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-    const int x0 = 2 * t;
-    if (x0 >= a.g.nx || y >= a.g.ny) return;
+    if (2 * t >= row_end<T, kRag>(a.g.nx) || y >= a.g.ny) return;
+    const PairCols<kRag> X(2 * t, a.g.nx);
+    const int x0 = X.x0, xm = X.xm, xp = X.xp;
+    const bool past = kRag && X.at != x0;
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
-    const int xm = (x0 == 0) ? a.g.nx - 1 : x0 - 1;
-    const int xp = (x0 + 2 == a.g.nx) ? 0 : x0 + 2;
     const int own = R.own + x0;
+    // rows along a wall take the wall selects, the others the plain accesses
+    // (see pull_pairs)
+    const bool edge = kWalls && (R.edge || blockDim.x < 32);
     f2 f[Q];
-    static_for<Q>([&](auto iq) {
-        constexpr int q = decltype(iq)::value;
-        constexpr int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
-        constexpr int o = opposite<Q>(q);
-        f2 v;
-        if (kWalls && R.wall[j][k]) {
-            v = Pair<T>::ld2(io.in[q] + own);
-        } else {
-            const T *row = io.in[o] + R.off[j][k];
-            if constexpr (i == 0)
-                v = Pair<T>::ld2(row + x0);
-            else if constexpr (i == 1)
-                v = f2(Pair<T>::ld1(row + xm), Pair<T>::ld1(row + x0));
+    const auto load = [&](auto sel) {
+        static_for<Q>([&](auto iq) {
+            constexpr int q = decltype(iq)::value;
+            constexpr int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
+            if (decltype(sel)::value && R.wall[j][k])
+                f[q] = Pair<T>::ld2(element<kRag, kPlain>(io.in[q], own));
             else
-                v = f2(Pair<T>::ld1(row + x0 + 1), Pair<T>::ld1(row + xp));
-        }
-        f[q] = v;
-    });
-    pair_inputs<Q, T, kWalls>(io, R, x0, xm, xp, f);
+                f[q] = ld_shifted<kPlain, kPlain && !kRag>(io.in[opposite<Q>(q)], R.off[j][k], i,
+                                                          X);
+        });
+    };
+    if (edge)
+        load(std::integral_constant<bool, kWalls>{});
+    else
+        load(std::false_type{});
+    pair_inputs<Q, T>(io, R, X, f);
     unsigned seed = 0;
     if constexpr (!kSeedAfterCollision<Q, T>) seed = pair_seed<Q>(f, own);
-    const float4 J = pair_collide<Q, T, kEq, kForce>(io, a, pr, x0, y, z, own, f);
+    const float4 J = pair_collide<Q, T, kEq, kForce>(io, a, pr, X, y, z, own, f);
     if constexpr (kSeedAfterCollision<Q, T>) seed = pair_seed<Q>(f, own);
-    static_for<Q>([&](auto iq) {
-        constexpr int q = decltype(iq)::value;
-        constexpr int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
-        constexpr int o = opposite<Q>(q);
-        const f2 v = stored_pair<Q, T, q>(f[q], store_scale<Q, T>(q), J);
-        // downstream neighbour x + e_q: the row of the mirrored pull
-        if (kWalls && R.wall[2 - j][2 - k]) {
-            Pair<T>::template st2s<q>(io.out[o] + own, v, seed);
-        } else {
-            T *row = io.out[q] + R.off[2 - j][2 - k];
-            if constexpr (i == 0)
-                Pair<T>::template st2s<q>(row + x0, v, seed);
-            else if constexpr (i == 1)
-                Pair<T>::template st1x2s<q>(row + x0 + 1, row + xp, v, seed);
-            else
-                Pair<T>::template st1x2s<q>(row + xm, row + x0, v, seed);
-        }
-    });
+    const auto store = [&](auto sel) {
+        static_for<Q>([&](auto iq) {
+            constexpr int q = decltype(iq)::value;
+            constexpr int i = ex<Q>(q), j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
+            constexpr int o = opposite<Q>(q);
+            const f2 v = stored_pair<Q, T, q>(f[q], store_scale<Q, T>(q), J);
+            // downstream neighbour x + e_q: the row of the mirrored pull
+            if (decltype(sel)::value && R.wall[2 - j][2 - k]) {
+                Pair<T>::template st2s<q>(element<kRag, kPlain>(io.out[o], R.own + X.at), v, seed);
+            } else {
+                const int row = R.off[2 - j][2 - k];
+                const auto dst = [&](int x) { return element<kRag, kPlain>(io.out[q], row + x); };
+                if constexpr (i == 0)
+                    Pair<T>::template st2s<q>(dst(X.at), v, seed);
+                else if constexpr (i == 1)
+                    Pair<T>::template st1x2s<q>(dst(past ? X.at : x0 + 1),
+                                                dst(past ? X.at + 1 : xp), v, seed);
+                else
+                    Pair<T>::template st1x2s<q>(dst(past ? X.at : xm), dst(past ? X.at + 1 : x0),
+                                                v, seed);
+            }
+        });
+    };
+    if (edge)
+        store(std::integral_constant<bool, kWalls>{});
+    else
+        store(std::false_type{});
 }
 
 // Initial state from FP64 density and velocity fields.
@@ -1230,77 +1299,113 @@ StepIO<T> read_io(const void *f, const Grid &g) {
     return step_io<Q, T>(f, nullptr, g, g.layout == kAASwapped ? 1 : 0);
 }
 
-// The two-cells-per-thread kernels serve grids with even nx (D3Q27 and
-// D3Q15); odd nx takes the one-cell kernel.
+// Launch geometry of the kernels with two cells per thread over `row` cells per
+// row (stored_row: to the end of the last sector).
+inline CellLaunch pair_launch(const Grid &g, int row) {
+    Grid half = g;
+    half.nx = (row + 1) / 2;
+    return cell_launch(half);
+}
+
+// Whether a grid takes the instantiations for ragged rows (kRag): rows that do
+// not fill their last sector, or planes beyond 32-bit byte offsets (element()).
+template <typename T>
+bool ragged(const Grid &g) {
+    return stored_row<T>(g.nx) != g.nx || g.pop * (long long)sizeof(T) > (1ll << 32);
+}
+
+// FP32 grids of odd rows up to this many cells take the one-cell step kernel.
+// us a step, one cell / two cells per thread / one-cell kernel before this one:
+// D3Q27 periodic 9^3 2.27 / 2.19 / 2.26, 17^3 2.33 / 2.51 / 2.20, 25^3 2.78 /
+// 2.64 / 2.82, 33^3 3.16 / 3.10 / 3.48; walled 9^3 2.26 / 2.78 / 2.57, 3 x 43 x 43
+// 2.78 / 3.74 / 3.03, 25^3 2.78 / 3.44 / 3.06, 33^3 3.80 / 3.22 / 3.99.
+constexpr long long kSmallCells = 8192, kSmallWalledCells = 20480;
+
+// kForm: the rate-1 relaxation (D3Q27), a force anywhere (D3Q15).
+template <int Q, typename T, bool kWalls, bool kForm>
+void launch_step_kernel(const StepIO<T> &io, const StepArgs &a, const PackedRates &pr,
+                      cudaStream_t st) {
+    if constexpr (std::is_same<T, float>::value) {
+        const long long cells = (long long)a.g.nx * a.g.ny * a.g.nz;
+        if (a.g.nx % 2 && cells <= (kWalls ? kSmallWalledCells : kSmallCells)) {
+            const CellLaunch L = cell_launch(a.g);
+            step1_kernel<Q, kWalls, kForm><<<L.grid, L.block, 0, st>>>(io, a);
+            return;
+        }
+    }
+    const CellLaunch L = pair_launch(a.g, stored_row<T>(a.g.nx));
+    // grids of short rows are small, and a second copy of the loads (pull_pairs)
+    // costs them more than it saves: D3Q27 FP32 between walls, 16^3 3.55 / 3.05
+    // us, 16 x 64 x 64 4.13 / 3.75 us with / without it
+    const bool is_short = L.block.x < 32 && !ragged<T>(a.g);
+    if constexpr (Q == 27) {
+        if constexpr (kWalls) {
+            if (is_short) {
+                step2_kernel<T, true, kForm, false, true><<<L.grid, L.block, 0, st>>>(io, a, pr);
+                return;
+            }
+        }
+        if (ragged<T>(a.g))
+            step2_kernel<T, kWalls, kForm, true><<<L.grid, L.block, 0, st>>>(io, a, pr);
+        else
+            step2_kernel<T, kWalls, kForm, false><<<L.grid, L.block, 0, st>>>(io, a, pr);
+    } else {
+        // (FP32 and FP16 the other way round: 16^3 2.27 / 2.47, 16 x 64 x 64 2.91 /
+        // 3.01 us with / without it; BF16 2.78 / 2.72)
+        if constexpr (kWalls && Storage<T>::kRef) {
+            if (is_short) {
+                step2_q15_kernel<T, true, kForm, false, true>
+                    <<<L.grid, L.block, 0, st>>>(io, a, pr);
+                return;
+            }
+        }
+        if (ragged<T>(a.g))
+            step2_q15_kernel<T, kWalls, kForm, true><<<L.grid, L.block, 0, st>>>(io, a, pr);
+        else
+            step2_q15_kernel<T, kWalls, kForm, false><<<L.grid, L.block, 0, st>>>(io, a, pr);
+    }
+}
+
+// Ragged rows (kRag) take their own instantiation of the two-cell kernels, so
+// that the others keep immediate offsets.
 template <int Q, typename T>
 cudaError_t launch_step(const void *fin, void *fout, const StepArgs &a, cudaStream_t st) {
     const StepIO<T> io = step_io<Q, T>(fin, fout, a.g);
     const bool walls = a.g.bc != 0;
     if constexpr (std::is_same<T, float>::value) {
-        if (a.sr32) {  // stochastically rounded FP32 update: the one-cell kernel, any nx
+        if (a.sr32) {
             const CellLaunch L = cell_launch(a.g);
             if (walls)
-                step_kernel<Q, T, true, true><<<L.grid, L.block, 0, st>>>(io, a);
+                step_sr32_kernel<Q, true><<<L.grid, L.block, 0, st>>>(io, a);
             else
-                step_kernel<Q, T, false, true><<<L.grid, L.block, 0, st>>>(io, a);
+                step_sr32_kernel<Q, false><<<L.grid, L.block, 0, st>>>(io, a);
             return cudaGetLastError();
         }
     }
-    if constexpr (Q == 27) {
-        if (a.g.nx % 2 == 0) {
-            Grid half = a.g;
-            half.nx = a.g.nx / 2;
-            const CellLaunch L = cell_launch(half);
-            const PackedRates pr = packed_rates(a, kFoldedLoad<27, T>());
-            const bool eq = higher_rates_are_one(a);
-            if (walls && eq)
-                step2_kernel<T, true, true><<<L.grid, L.block, 0, st>>>(io, a, pr);
-            else if (walls)
-                step2_kernel<T, true, false><<<L.grid, L.block, 0, st>>>(io, a, pr);
-            else if (eq)
-                step2_kernel<T, false, true><<<L.grid, L.block, 0, st>>>(io, a, pr);
-            else
-                step2_kernel<T, false, false><<<L.grid, L.block, 0, st>>>(io, a, pr);
-            return cudaGetLastError();
-        }
-    } else {
-        if (a.g.nx % 2 == 0) {
-            Grid half = a.g;
-            half.nx = a.g.nx / 2;
-            const CellLaunch L = cell_launch(half);
-            const PackedRates pr = packed_rates(a);
-            if (walls && a.has_force)
-                step2_q15_kernel<T, true, true><<<L.grid, L.block, 0, st>>>(io, a, pr);
-            else if (walls)
-                step2_q15_kernel<T, true, false><<<L.grid, L.block, 0, st>>>(io, a, pr);
-            else if (a.has_force)
-                step2_q15_kernel<T, false, true><<<L.grid, L.block, 0, st>>>(io, a, pr);
-            else
-                step2_q15_kernel<T, false, false><<<L.grid, L.block, 0, st>>>(io, a, pr);
-            return cudaGetLastError();
-        }
-    }
-    {
-        const CellLaunch L = cell_launch(a.g);
-        if (walls)
-            step_kernel<Q, T, true><<<L.grid, L.block, 0, st>>>(io, a);
-        else
-            step_kernel<Q, T, false><<<L.grid, L.block, 0, st>>>(io, a);
-    }
+    const PackedRates pr = packed_rates(a, kFoldedLoad<Q, T>());
+    const bool form = Q == 27 ? higher_rates_are_one(a) : a.has_force != 0;
+    if (walls && form)
+        launch_step_kernel<Q, T, true, true>(io, a, pr, st);
+    else if (walls)
+        launch_step_kernel<Q, T, true, false>(io, a, pr, st);
+    else if (form)
+        launch_step_kernel<Q, T, false, true>(io, a, pr, st);
+    else
+        launch_step_kernel<Q, T, false, false>(io, a, pr, st);
     return cudaGetLastError();
 }
 
-template <int Q, typename T, bool kEq, bool kForce>
+template <int Q, typename T, bool kEq, bool kForce, bool kRag>
 void launch_aa_kernels(const StepIO<T> &io, const StepArgs &a, const PackedRates &pr, bool even,
                        const CellLaunch &L, cudaStream_t st) {
     if (even && a.g.bc)
-        aa_even_kernel<Q, T, true, kEq, kForce><<<L.grid, L.block, 0, st>>>(io, a, pr);
+        aa_even_kernel<Q, T, true, kEq, kForce, kRag><<<L.grid, L.block, 0, st>>>(io, a, pr);
     else if (even)
-        aa_even_kernel<Q, T, false, kEq, kForce><<<L.grid, L.block, 0, st>>>(io, a, pr);
+        aa_even_kernel<Q, T, false, kEq, kForce, kRag><<<L.grid, L.block, 0, st>>>(io, a, pr);
     else if (a.g.bc)
-        aa_odd_kernel<Q, T, true, kEq, kForce><<<L.grid, L.block, 0, st>>>(io, a, pr);
+        aa_odd_kernel<Q, T, true, kEq, kForce, kRag><<<L.grid, L.block, 0, st>>>(io, a, pr);
     else
-        aa_odd_kernel<Q, T, false, kEq, kForce><<<L.grid, L.block, 0, st>>>(io, a, pr);
+        aa_odd_kernel<Q, T, false, kEq, kForce, kRag><<<L.grid, L.block, 0, st>>>(io, a, pr);
 }
 
 // One in-place (AA) step on buffer buf: even (kAANatural -> kAASwapped) or
@@ -1311,21 +1416,20 @@ template <int Q, typename T>
 cudaError_t launch_step_aa(void *buf, const StepArgs &a, bool even, cudaStream_t st) {
     // BF16 references: array 0 for the natural layout, 1 for the swapped one
     const StepIO<T> io = step_io<Q, T>(buf, buf, a.g, even ? 0 : 1, even ? 1 : 0);
-    Grid half = a.g;
-    half.nx = a.g.nx / 2;
-    const CellLaunch L = cell_launch(half);
+    const CellLaunch L = pair_launch(a.g, stored_row<T>(a.g.nx));
     const PackedRates pr = packed_rates(a, kFoldedLoad<Q, T>());
-    if constexpr (Q == 27) {
-        if (higher_rates_are_one(a))
-            launch_aa_kernels<Q, T, true, true>(io, a, pr, even, L, st);
+    const auto launch = [&](auto form) {
+        constexpr bool kEq = Q == 27 && decltype(form)::value;
+        constexpr bool kForce = Q == 27 || decltype(form)::value;
+        if (ragged<T>(a.g))
+            launch_aa_kernels<Q, T, kEq, kForce, true>(io, a, pr, even, L, st);
         else
-            launch_aa_kernels<Q, T, false, true>(io, a, pr, even, L, st);
-    } else {
-        if (a.has_force)
-            launch_aa_kernels<Q, T, false, true>(io, a, pr, even, L, st);
-        else
-            launch_aa_kernels<Q, T, false, false>(io, a, pr, even, L, st);
-    }
+            launch_aa_kernels<Q, T, kEq, kForce, false>(io, a, pr, even, L, st);
+    };
+    if (Q == 27 ? higher_rates_are_one(a) : a.has_force != 0)
+        launch(std::true_type{});
+    else
+        launch(std::false_type{});
     return cudaGetLastError();
 }
 
@@ -1333,9 +1437,7 @@ cudaError_t launch_step_aa(void *buf, const StepArgs &a, bool even, cudaStream_t
 template <int Q, typename T>
 cudaError_t launch_ref_init(T *buf, const Grid &g, const double *u, const double *f,
                             cudaStream_t st) {
-    Grid half = g;
-    half.nx = (g.nx + 1) / 2;
-    const CellLaunch L = cell_launch(half);
+    const CellLaunch L = pair_launch(g, g.nx);
     ref_init_kernel<Q, T><<<L.grid, L.block, 0, st>>>(buf, g, u, f);
     return cudaGetLastError();
 }

@@ -226,19 +226,6 @@ __device__ __forceinline__ void store_dev(T *p, int a, float dev, float ref = 0.
         Storage<T>::store(p, dev);
 }
 
-// The step's store of population a of one cell: FP32 as is, 16-bit
-// stochastically rounded (ref: as for store_dev).
-template <int Q, typename T, int a>
-__device__ __forceinline__ void store_dev_step(T *p, float dev, unsigned seed, float ref = 0.0f) {
-    if constexpr (Storage<T>::kScaled) {
-        const unsigned d =
-            pack_sr<T, a>(fmaf(dev, float(1.0 / weight<Q>(a)), -ref), 0.0f, seed);
-        __stcs(reinterpret_cast<unsigned short *>(p), static_cast<unsigned short>(d & 0xffffu));
-    } else {
-        Storage<T>::store(p, dev);
-    }
-}
-
 // ---------------------------------------------------------------------- grid
 // How a state buffer holds the pre-collision distributions f(x, t):
 //   kPull:      post-collision values of the previous step at their own cells
