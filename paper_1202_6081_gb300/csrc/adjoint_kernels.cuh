@@ -18,13 +18,14 @@
 namespace lbm {
 
 // Per-cell reverse of the collision, chosen by the lattice (array size).
-template <typename V>
+// kEq: the rate-1 form (D3Q27).
+template <bool kEq, typename V>
 __device__ __forceinline__ void adjoint_collide(const V (&f)[27], V Fx, V Fy, V Fz,
                                                 const Rates27<V> &r, const V (&mu)[27],
                                                 V (&lam)[27], V &gx, V &gy, V &gz) {
-    adjoint27<V>(f, Fx, Fy, Fz, r, mu, lam, gx, gy, gz);
+    adjoint27<kEq, V>(f, Fx, Fy, Fz, r, mu, lam, gx, gy, gz);
 }
-template <typename V>
+template <bool, typename V>
 __device__ __forceinline__ void adjoint_collide(const V (&f)[15], V Fx, V Fy, V Fz,
                                                 const Rates15<V> &r, const V (&mu)[15],
                                                 V (&lam)[15], V &gx, V &gy, V &gz) {
@@ -78,13 +79,19 @@ __device__ __forceinline__ void pull_adjoint(const AdjointArgs &g, const Rows<kW
 // packed f32x2 arithmetic.  The state is pulled as in step2_kernel; the adjoint
 // is pulled from the mirrored neighbours x + e_q: for e_x = 0 an aligned pair,
 // for e_x = +1 the cells (x0 + 1, x0 + 2), for e_x = -1 (x0 - 1, x0).
-// 3 blocks of 128 threads per SM: 168 registers.  D3Q27 spills a few of its
-// 242 there but beats 2 blocks and 4 (128 registers, ~700 B of spills:
-// 0.206 vs 0.135 ms at 128^3); D3Q15 fits without spills and beats 4 blocks
-// (276 B of spills; 0.098 vs 0.090 ms).
+// Bound by HBM: 360 bytes per cell (D3Q27 FP32 with a force field and dJ/dF).
+// 3 blocks of 128 threads per SM, 168 registers: D3Q15 fits without spills;
+// D3Q27 at general rates spills ~100 B (121 us at 128^3; 4 blocks spill ~700 B,
+// 206 us).  The rate-1 form (kEq, adjoint27) needs fewer and takes 4 blocks, 128
+// registers: 128^3 in 113.8 us, 6.64 TB/s, where the general form took 135; FP16
+// states 114 / 119 us at 4 / 3 blocks; 3 blocks for BF16 states (117 / 126 at 4)
+// and ragged rows (126 x 128 x 128 walled 121 / 130).
 // kRag: ragged rows (PairCols).
-template <int Q, typename T, bool kWalls, bool kRag>
-__global__ void __launch_bounds__(128, 3) adjoint2_kernel(const StepIO<T> io, const AdjointArgs g,
+template <typename T, bool kRag, bool kEq>
+constexpr int kAdjointBlocks = kEq && !kRag && !Storage<T>::kRef ? 4 : 3;
+
+template <int Q, typename T, bool kWalls, bool kRag, bool kEq>
+__global__ void __launch_bounds__(128, (kAdjointBlocks<T, kRag, kEq>)) adjoint2_kernel(const StepIO<T> io, const AdjointArgs g,
                                                        const StepArgs a, const PackedRates pr) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
@@ -121,7 +128,7 @@ __global__ void __launch_bounds__(128, 3) adjoint2_kernel(const StepIO<T> io, co
     }
     const typename PairRates<Q>::type r = PairRates<Q>::load(pr);
     f2 lam[Q], gF[3];
-    adjoint_collide<f2>(f, Fx, Fy, Fz, r, mu, lam, gF[0], gF[1], gF[2]);
+    adjoint_collide<kEq, f2>(f, Fx, Fy, Fz, r, mu, lam, gF[0], gF[1], gF[2]);
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         Pair<float>::st2(element<kRag>(g.lam_out[q], R.own + X.at), lam[q]);
@@ -241,12 +248,22 @@ cudaError_t launch_adjoint(const void *f_t, const float *lam_next, float *lam_ou
     g.gF = gF;
     const CellLaunch L = pair_launch(a.g, stored_row<float>(a.g.nx));
     const PackedRates pr = packed_rates(a);
-    if (ragged<float>(a.g))  // one instantiation, with the wall selects: the rarer case
-        adjoint2_kernel<Q, T, true, true><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
-    else if (a.g.bc)
-        adjoint2_kernel<Q, T, true, false><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
-    else
-        adjoint2_kernel<Q, T, false, false><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
+    const auto launch = [&](auto eq) {
+        constexpr bool kEq = decltype(eq)::value;
+        if (ragged<float>(a.g))  // one form, with the wall selects: the rarer case
+            adjoint2_kernel<Q, T, true, true, kEq><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
+        else if (a.g.bc)
+            adjoint2_kernel<Q, T, true, false, kEq><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
+        else
+            adjoint2_kernel<Q, T, false, false, kEq><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
+    };
+    if constexpr (Q == 27) {
+        if (higher_rates_are_one(a)) {
+            launch(std::true_type{});
+            return cudaGetLastError();
+        }
+    }
+    launch(std::false_type{});
     return cudaGetLastError();
 }
 

@@ -86,7 +86,11 @@ __device__ __forceinline__ void shift_u_terms(const V (&Db)[3][3][3], const V (&
 // Reverse of relax27.  Dt: post-collision moments (forward output); Db: on
 // input the adjoint of Dt, on output the adjoint of the pre-relaxation D.
 // Accumulates the adjoints of u and drho.
-template <typename V>
+// kEq (as in relax27): the rates from the trace on are all 1, so the adjoints
+// of those pre-relaxation moments are 0 -- they are left unwritten, for the
+// caller not to read -- and their attractors take the post-collision adjoints
+// as they are.
+template <bool kEq, typename V>
 __device__ __forceinline__ void relax27_T(const V (&Dt)[3][3][3], V (&Db)[3][3][3], V ux, V uy,
                                           V uz, const Rates27<V> &r, V &gux, V &guy, V &guz,
                                           V &gdrho) {
@@ -97,14 +101,17 @@ __device__ __forceinline__ void relax27_T(const V (&Dt)[3][3][3], V (&Db)[3][3][
     const V Kwx = third + ux2, Kwy = third + uy2, Kwz = third + uz2;
     const V dxx = Dt[2][0][0], dyy = Dt[0][2][0], dzz = Dt[0][0][2];
     V gKx = zero, gKy = zero, gKz = zero;                 // adjoints of Kw_i
+    const auto to_attractor = [&](int b, V g) { return kEq ? g : r.w[b] * g; };
+    const auto keep = [&](int b, V &d) {
+        if constexpr (!kEq) d = r.omw[b] * d;
+    };
     V gdx = Db[2][0][0], gdy = Db[0][2][0], gdz = Db[0][0][2];  // of dxx, dyy, dzz
 
     // order 6: dK = kt_x kt_y kt_z - Kw_x Kw_y Kw_z
     {
         const V ktx = Kwx + dxx, kty = Kwy + dyy, ktz = Kwz + dzz;
-        const V g = Db[2][2][2];
-        Db[2][2][2] = r.omw[26] * g;
-        const V gK = r.w[26] * g;
+        const V gK = to_attractor(26, Db[2][2][2]);
+        keep(26, Db[2][2][2]);
         gdx = vfma(kty * ktz, gK, gdx);
         gdy = vfma(ktx * ktz, gK, gdy);
         gdz = vfma(ktx * kty, gK, gdz);
@@ -115,64 +122,57 @@ __device__ __forceinline__ void relax27_T(const V (&Dt)[3][3][3], V (&Db)[3][3][
     }
     // order 5
     {
-        V g = Db[1][2][2];
-        Db[1][2][2] = r.omw[23] * g;
-        g = r.w[23] * g;
+        V g = to_attractor(23, Db[1][2][2]);
+        keep(23, Db[1][2][2]);
         gux = vfma(Kwy * Kwz, g, gux);
         gKy = vfma(ux * Kwz, g, gKy);
         gKz = vfma(ux * Kwy, g, gKz);
-        g = Db[2][1][2];
-        Db[2][1][2] = r.omw[24] * g;
-        g = r.w[24] * g;
+        g = to_attractor(24, Db[2][1][2]);
+        keep(24, Db[2][1][2]);
         guy = vfma(Kwx * Kwz, g, guy);
         gKx = vfma(uy * Kwz, g, gKx);
         gKz = vfma(uy * Kwx, g, gKz);
-        g = Db[2][2][1];
-        Db[2][2][1] = r.omw[25] * g;
-        g = r.w[25] * g;
+        g = to_attractor(25, Db[2][2][1]);
+        keep(25, Db[2][2][1]);
         guz = vfma(Kwx * Kwy, g, guz);
         gKx = vfma(uz * Kwy, g, gKx);
         gKy = vfma(uz * Kwx, g, gKy);
     }
     // order 4, mixed: D~ = omw D + nw Kw_i u_j u_k
     {
-        V g = Db[2][1][1];
-        Db[2][1][1] = r.omw[20] * g;
-        g = r.nw[20] * g;
+        V g = r.nw[20] * Db[2][1][1];
+        keep(20, Db[2][1][1]);
         gKx = vfma(uy * uz, g, gKx);
         guy = vfma(Kwx * uz, g, guy);
         guz = vfma(Kwx * uy, g, guz);
-        g = Db[1][2][1];
-        Db[1][2][1] = r.omw[21] * g;
-        g = r.nw[21] * g;
+        g = r.nw[21] * Db[1][2][1];
+        keep(21, Db[1][2][1]);
         gKy = vfma(ux * uz, g, gKy);
         gux = vfma(Kwy * uz, g, gux);
         guz = vfma(Kwy * ux, g, guz);
-        g = Db[1][1][2];
-        Db[1][1][2] = r.omw[22] * g;
-        g = r.nw[22] * g;
+        g = r.nw[22] * Db[1][1][2];
+        keep(22, Db[1][1][2]);
         gKz = vfma(ux * uy, g, gKz);
         gux = vfma(Kwz * uy, g, gux);
         guy = vfma(Kwz * ux, g, guy);
     }
     // order 4, diagonal: A = xxyy, B = xxzz, C = yyzz
     {
-        const V gABn = half * (Db[2][2][0] + Db[2][0][2]);
-        const V g19 = half * (Db[2][2][0] - Db[2][0][2]);
-        const V g17 = third * vfma(two, gABn, Db[0][2][2]);
-        const V g18 = third * (gABn - Db[0][2][2]);
-        {
+        V gA = Db[2][2][0], gB = Db[2][0][2], gC = Db[0][2][2];
+        if constexpr (!kEq) {
+            const V gABn = half * (gA + gB), g19 = half * (gA - gB);
+            const V g17 = third * vfma(two, gABn, gC), g18 = third * (gABn - gC);
             const V a17 = r.omw[17] * g17, a18 = r.omw[18] * g18, a19 = r.omw[19] * g19;
-            const V t = a17 + a18;
-            Db[2][2][0] = t + a19;
-            Db[2][0][2] = t - a19;
+            const V ta = a17 + a18;
+            Db[2][2][0] = ta + a19;
+            Db[2][0][2] = ta - a19;
             Db[0][2][2] = a17 - (a18 + a18);
+            const V b17 = r.w[17] * g17, b18 = r.w[18] * g18, b19 = r.w[19] * g19;
+            const V tb = b17 + b18;
+            gA = tb + b19;
+            gB = tb - b19;
+            gC = b17 - (b18 + b18);
         }
-        const V b17 = r.w[17] * g17, b18 = r.w[18] * g18, b19 = r.w[19] * g19;
-        const V t = b17 + b18;
-        const V gA = t + b19;
-        const V gB = t - b19;
-        const V gC = b17 - (b18 + b18);
         // dA = Kwx dyy + Kwy dxx + dxx dyy, etc.
         const V kx = Kwx + dxx, ky = Kwy + dyy, kz = Kwz + dzz;
         gdx = vfma(ky, gA, vfma(kz, gB, gdx));
@@ -184,42 +184,53 @@ __device__ __forceinline__ void relax27_T(const V (&Dt)[3][3][3], V (&Db)[3][3][
     }
     // order 3
     {
-        const V gs = half * (Db[1][2][0] + Db[1][0][2]);
-        const V gt = half * (Db[1][2][0] - Db[1][0][2]);
-        const V as = r.w[10] * gs, at = r.w[13] * gt;
-        gux = vfma(as, Kwy + Kwz, vfma(at, Kwy - Kwz, gux));
-        gKy = vfma(ux, as + at, gKy);
-        gKz = vfma(ux, as - at, gKz);
-        const V bs = r.omw[10] * gs, bt = r.omw[13] * gt;
-        Db[1][2][0] = bs + bt;
-        Db[1][0][2] = bs - bt;
+        V g1 = Db[1][2][0], g2 = Db[1][0][2];
+        if constexpr (!kEq) {
+            const V gs = half * (g1 + g2), gt = half * (g1 - g2);
+            const V as = r.w[10] * gs, at = r.w[13] * gt;
+            const V bs = r.omw[10] * gs, bt = r.omw[13] * gt;
+            Db[1][2][0] = bs + bt;
+            Db[1][0][2] = bs - bt;
+            g1 = as + at;
+            g2 = as - at;
+        }
+        gux = vfma(g1, Kwy, vfma(g2, Kwz, gux));
+        gKy = vfma(ux, g1, gKy);
+        gKz = vfma(ux, g2, gKz);
     }
     {
-        const V gs = half * (Db[2][1][0] + Db[0][1][2]);
-        const V gt = half * (Db[2][1][0] - Db[0][1][2]);
-        const V as = r.w[11] * gs, at = r.w[14] * gt;
-        guy = vfma(as, Kwx + Kwz, vfma(at, Kwx - Kwz, guy));
-        gKx = vfma(uy, as + at, gKx);
-        gKz = vfma(uy, as - at, gKz);
-        const V bs = r.omw[11] * gs, bt = r.omw[14] * gt;
-        Db[2][1][0] = bs + bt;
-        Db[0][1][2] = bs - bt;
+        V g1 = Db[2][1][0], g2 = Db[0][1][2];
+        if constexpr (!kEq) {
+            const V gs = half * (g1 + g2), gt = half * (g1 - g2);
+            const V as = r.w[11] * gs, at = r.w[14] * gt;
+            const V bs = r.omw[11] * gs, bt = r.omw[14] * gt;
+            Db[2][1][0] = bs + bt;
+            Db[0][1][2] = bs - bt;
+            g1 = as + at;
+            g2 = as - at;
+        }
+        guy = vfma(g1, Kwx, vfma(g2, Kwz, guy));
+        gKx = vfma(uy, g1, gKx);
+        gKz = vfma(uy, g2, gKz);
     }
     {
-        const V gs = half * (Db[2][0][1] + Db[0][2][1]);
-        const V gt = half * (Db[2][0][1] - Db[0][2][1]);
-        const V as = r.w[12] * gs, at = r.w[15] * gt;
-        guz = vfma(as, Kwx + Kwy, vfma(at, Kwx - Kwy, guz));
-        gKx = vfma(uz, as + at, gKx);
-        gKy = vfma(uz, as - at, gKy);
-        const V bs = r.omw[12] * gs, bt = r.omw[15] * gt;
-        Db[2][0][1] = bs + bt;
-        Db[0][2][1] = bs - bt;
+        V g1 = Db[2][0][1], g2 = Db[0][2][1];
+        if constexpr (!kEq) {
+            const V gs = half * (g1 + g2), gt = half * (g1 - g2);
+            const V as = r.w[12] * gs, at = r.w[15] * gt;
+            const V bs = r.omw[12] * gs, bt = r.omw[15] * gt;
+            Db[2][0][1] = bs + bt;
+            Db[0][2][1] = bs - bt;
+            g1 = as + at;
+            g2 = as - at;
+        }
+        guz = vfma(g1, Kwx, vfma(g2, Kwy, guz));
+        gKx = vfma(uz, g1, gKx);
+        gKy = vfma(uz, g2, gKy);
     }
     {
-        const V g = Db[1][1][1];
-        Db[1][1][1] = r.omw[16] * g;
-        const V a = r.w[16] * g;
+        const V a = to_attractor(16, Db[1][1][1]);
+        keep(16, Db[1][1][1]);
         gux = vfma(uy * uz, a, gux);
         guy = vfma(ux * uz, a, guy);
         guz = vfma(ux * uy, a, guz);
@@ -248,13 +259,14 @@ __device__ __forceinline__ void relax27_T(const V (&Dt)[3][3][3], V (&Db)[3][3][
         const V ga = half * (gdx - gdy);
         const V gb = vfma(nthird, gdz, sixth * sxy);
         const V gc = third * (sxy + gdz);
-        const V a7 = r.nw[7] * ga, a8 = r.nw[8] * gb, a9 = r.w[9] * gc;
+        const V a7 = r.nw[7] * ga, a8 = r.nw[8] * gb, a9 = to_attractor(9, gc);
         gux = vfma(ux + ux, (a7 + a8) - a9, gux);
         guy = vfma(uy + uy, (a8 - a7) - a9, guy);
         guz = guz - (uz + uz) * ((a8 + a8) + a9);
         gdrho = gdrho + a9;
-        const V ba = r.omw[7] * ga, bb = r.omw[8] * gb, bc = r.omw[9] * gc;
-        const V t = bb + bc;
+        const V ba = r.omw[7] * ga, bb = r.omw[8] * gb;
+        const V bc = kEq ? zero : r.omw[9] * gc;
+        const V t = kEq ? bb : bb + bc;
         Db[2][0][0] = t + ba;
         Db[0][2][0] = t - ba;
         Db[0][0][2] = bc - (bb + bb);
@@ -269,7 +281,11 @@ __device__ __forceinline__ void relax27_T(const V (&Dt)[3][3][3], V (&Db)[3][3][
 // pre-collision deviations (slot order); mu: adjoint of the post-collision
 // values (slot order).  Writes lam (slot order) and the force adjoint
 // (gFx, gFy, gFz).
-template <typename V>
+// kEq: the rates from the trace on are all 1 (relax27).  Then the adjoints of
+// the moments of order >= 3 end at the relaxation: of the pre-collision state
+// only its moments up to order 2 enter, and lam is a polynomial of degree 2 in
+// the velocity with 10 coefficients instead of 27.
+template <bool kEq, typename V>
 __device__ __forceinline__ void adjoint27(const V (&f)[27], V Fx, V Fy, V Fz,
                                           const Rates27<V> &r, const V (&mu)[27], V (&lam)[27],
                                           V &gFx, V &gFy, V &gFz) {
@@ -288,7 +304,7 @@ __device__ __forceinline__ void adjoint27(const V (&f)[27], V Fx, V Fy, V Fz,
     Dt[1][0][0] = Dt[1][0][0] + Fx;
     Dt[0][1][0] = Dt[0][1][0] + Fy;
     Dt[0][0][1] = Dt[0][0][1] + Fz;
-    relax27<V>(Dt, ux, uy, uz, drho, r);
+    relax27<V, kEq>(Dt, ux, uy, uz, drho, r);
 
     // ---- reverse of the inverse sweeps: Db = Inv(u)^T mu (x, then y, then z)
     V Db[3][3][3];
@@ -318,38 +334,62 @@ __device__ __forceinline__ void adjoint27(const V (&f)[27], V Fx, V Fy, V Fz,
     shift_u_terms(Db, Dt, gux, guy, guz);
     V gdrho = zero;
     // ---- reverse of the relaxation
-    relax27_T(Dt, Db, ux, uy, uz, r, gux, guy, guz, gdrho);
+    relax27_T<kEq>(Dt, Db, ux, uy, uz, r, gux, guy, guz, gdrho);
     // ---- source: D = K + sigma(F)
     gFx = Db[1][0][0];
     gFy = Db[0][1][0];
     gFz = Db[0][0][1];
-    // ---- u through Shift(u): -<Kbar, N K>
-    {
-        V sx, sy, sz;
-        shift_u_terms(Db, K, sx, sy, sz);
-        gux = gux - sx;
-        guy = guy - sy;
-        guz = guz - sz;
-    }
-    // ---- reverse of the shifts: Rbar = Shift(u)^T Kbar (z, y, x; they commute)
-    {
-        const V nux = zero - ux, nuy = zero - uy, nuz = zero - uz;
-        const V nux2 = nux + nux, nuy2 = nuy + nuy, nuz2 = nuz + nuz;
+    const V nux = zero - ux, nuy = zero - uy, nuz = zero - uz;
+    if constexpr (kEq) {
+        // ---- u through Shift(u): -<Kbar, N K>, orders <= 2
+        const V two = splat<V>(2.0f);
+        const V x = vfma(Db[1][0][0], K[0][0][0],
+                         vfma(Db[1][1][0], K[0][1][0], Db[1][0][1] * K[0][0][1]));
+        const V y = vfma(Db[0][1][0], K[0][0][0],
+                         vfma(Db[1][1][0], K[1][0][0], Db[0][1][1] * K[0][0][1]));
+        const V z = vfma(Db[0][0][1], K[0][0][0],
+                         vfma(Db[1][0][1], K[1][0][0], Db[0][1][1] * K[0][1][0]));
+        gux = gux - vfma(two * Db[2][0][0], K[1][0][0], x);
+        guy = guy - vfma(two * Db[0][2][0], K[0][1][0], y);
+        guz = guz - vfma(two * Db[0][0][2], K[0][0][1], z);
+        // ---- reverse of the shifts, orders <= 2
+        const V tx = vfma(nuy, Db[1][1][0], vfma(nuz, Db[1][0][1], Db[1][0][0]));
+        const V ty = vfma(nuz, Db[0][1][1], Db[0][1][0]);
+        Db[0][0][0] = vfma(nux, vfma(nux, Db[2][0][0], tx),
+                           vfma(nuy, vfma(nuy, Db[0][2][0], ty),
+                                vfma(nuz, vfma(nuz, Db[0][0][2], Db[0][0][1]), Db[0][0][0])));
+        Db[1][0][0] = vfma(nux + nux, Db[2][0][0], tx);
+        Db[0][1][0] = vfma(nuy + nuy, Db[0][2][0], vfma(nux, Db[1][1][0], ty));
+        Db[0][0][1] = vfma(nuz + nuz, Db[0][0][2],
+                           vfma(nux, Db[1][0][1], vfma(nuy, Db[0][1][1], Db[0][0][1])));
+    } else {
+        // ---- u through Shift(u): -<Kbar, N K>
+        {
+            V sx, sy, sz;
+            shift_u_terms(Db, K, sx, sy, sz);
+            gux = gux - sx;
+            guy = guy - sy;
+            guz = guz - sz;
+        }
+        // ---- reverse of the shifts: Rbar = Shift(u)^T Kbar (z, y, x; they commute)
+        {
+            const V nux2 = nux + nux, nuy2 = nuy + nuy, nuz2 = nuz + nuz;
 #pragma unroll
-        for (int m = 0; m < 3; ++m)
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int n = 0; n < 3; ++n)
+                    shift_line_T(nuz, nuz2, Db[m][n][0], Db[m][n][1], Db[m][n][2]);
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+                    shift_line_T(nuy, nuy2, Db[m][0][p], Db[m][1][p], Db[m][2][p]);
 #pragma unroll
             for (int n = 0; n < 3; ++n)
-                shift_line_T(nuz, nuz2, Db[m][n][0], Db[m][n][1], Db[m][n][2]);
 #pragma unroll
-        for (int m = 0; m < 3; ++m)
-#pragma unroll
-            for (int p = 0; p < 3; ++p)
-                shift_line_T(nuy, nuy2, Db[m][0][p], Db[m][1][p], Db[m][2][p]);
-#pragma unroll
-        for (int n = 0; n < 3; ++n)
-#pragma unroll
-            for (int p = 0; p < 3; ++p)
-                shift_line_T(nux, nux2, Db[0][n][p], Db[1][n][p], Db[2][n][p]);
+                for (int p = 0; p < 3; ++p)
+                    shift_line_T(nux, nux2, Db[0][n][p], Db[1][n][p], Db[2][n][p]);
+        }
     }
     // ---- u = (j + F/2) / rho
     const V inv_rho = vrcp(splat<V>(1.0f) + drho);
@@ -362,24 +402,45 @@ __device__ __forceinline__ void adjoint27(const V (&f)[27], V Fx, V Fy, V Fz,
     Db[1][0][0] = Db[1][0][0] + gjx;
     Db[0][1][0] = Db[0][1][0] + gjy;
     Db[0][0][1] = Db[0][0][1] + gjz;
-    // ---- reverse of the raw sums: lam = Sums^T Rbar
+    if constexpr (kEq) {
+        // ---- lam(e) = R000 + e . R1 + sum_ij e_i e_j R2
+        const V s0 = Db[0][0][0], s02 = s0 + Db[0][2][0];
+        const V S[3] = {s02 - Db[0][1][0], s0, s02 + Db[0][1][0]};                        // e_y
+        const V C[3] = {Db[0][0][1] - Db[0][1][1], Db[0][0][1], Db[0][0][1] + Db[0][1][1]};
+        const V B[3] = {Db[1][0][0] - Db[1][1][0], Db[1][0][0], Db[1][0][0] + Db[1][1][0]};
 #pragma unroll
-    for (int m = 0; m < 3; ++m)
+        for (int j = 0; j < 3; ++j) {
+            const V Sz = S[j] + Db[0][0][2];
+            const V even[3] = {Sz - C[j], S[j], Sz + C[j]};                               // e_z
+            const V odd[3] = {B[j] - Db[1][0][1], B[j], B[j] + Db[1][0][1]};
 #pragma unroll
-        for (int n = 0; n < 3; ++n) sums_line_T(Db[m][n][0], Db[m][n][1], Db[m][n][2]);
-#pragma unroll
-    for (int m = 0; m < 3; ++m)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) sums_line_T(Db[m][0][k], Db[m][1][k], Db[m][2][k]);
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            sums_line_T(Db[0][j][k], Db[1][j][k], Db[2][j][k]);
-            lam[s27(0, j, k)] = Db[0][j][k];
-            lam[s27(1, j, k)] = Db[1][j][k];
-            lam[s27(2, j, k)] = Db[2][j][k];
+            for (int k = 0; k < 3; ++k) {
+                const V e2 = even[k] + Db[2][0][0];
+                lam[s27(0, j, k)] = e2 - odd[k];
+                lam[s27(1, j, k)] = even[k];
+                lam[s27(2, j, k)] = e2 + odd[k];
+            }
         }
+    } else {
+        // ---- reverse of the raw sums: lam = Sums^T Rbar
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+#pragma unroll
+            for (int n = 0; n < 3; ++n) sums_line_T(Db[m][n][0], Db[m][n][1], Db[m][n][2]);
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) sums_line_T(Db[m][0][k], Db[m][1][k], Db[m][2][k]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                sums_line_T(Db[0][j][k], Db[1][j][k], Db[2][j][k]);
+                lam[s27(0, j, k)] = Db[0][j][k];
+                lam[s27(1, j, k)] = Db[1][j][k];
+                lam[s27(2, j, k)] = Db[2][j][k];
+            }
+    }
 }
 
 }  // namespace lbm
