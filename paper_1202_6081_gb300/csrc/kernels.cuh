@@ -1068,10 +1068,13 @@ __global__ void __launch_bounds__(128) set_state_kernel(const StepIO<T> io, cons
     if (!cell_coords(g, x, y, z)) return;
     const long long N = (long long)g.nx * g.ny * g.nz;
     const double *src = fin + dense_index(g, x, y, z);
+    double v[Q];  // all loads before the conversions, whose branches would order them
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[q] = __ldcs(src + q * N);
     float f[Q];
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
-        f[q] = deviation<Q, q>(__ldcs(src + q * N));
+        f[q] = deviation<Q, q>(v[q]);
     });
     scatter_state<Q, T>(io, g, x, y, z, f);
 }
