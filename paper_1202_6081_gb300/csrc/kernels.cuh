@@ -774,20 +774,19 @@ __device__ __forceinline__ void pair_force(const StepArgs &a, const PairCols<kRa
 // the collision in packed f32x2 arithmetic.  Loads of
 // populations with e_x = 0 and all stores are aligned 2-element accesses;
 // e_x = +-1 sources are two single loads (x0 - 1, x0) or (x0 + 1, x0 + 2).
-// Blocks of 128 per SM, by measurement: FP32 storage 5 (96 registers, no
-// spills; 6 blocks ran the same, 32.20k vs 32.23k MLUPS at 256^3, and 7
-// slower); 16-bit storage 6 (80 registers): with the rate-1 relaxation FP16
-// 48.2k / 48.0k MLUPS at 6 / 7 blocks at 512^3 (before it 41.2k / 44.3k /
-// 37.5k at 5 / 6 / 7), BF16 with its reference loads 38.6k / 39.4k at 5 / 6.
-template <typename T>
-constexpr int kStep2Blocks = Storage<T>::kScaled ? 6 : 5;
+// Blocks of 128 per SM, by measurement (us a step at 256^3): FP32 storage 5 (518;
+// 6: 523).  FP16 6 (327 / 326 / 323 at 6 / 5 / 7 blocks at the rate-1 form, at
+// 512^3 2642 / 2653 at 6 / 7; general rates 372 / 392 at 6 / 7).  BF16 with its
+// reference loads 5 (388.6 / 391.8 / 414 at 5 / 6 / 7; 32^3 2.91 / 3.10 at 5 / 6),
+// with the wall selects 6 (401 / 426 at 6 / 5).
+template <typename T, bool kWalls>
+constexpr int kStep2Blocks = Storage<T>::kScaled && (kWalls || !Storage<T>::kRef) ? 6 : 5;
 
 // kEq: the rates from the trace on are all 1 (relax27).
 // kShort: see pull_pairs.
 template <typename T, bool kWalls, bool kEq, bool kRag, bool kShort = false>
-__global__ void __launch_bounds__(128, kStep2Blocks<T>) step2_kernel(const StepIO<T> io,
-                                                                  const StepArgs a,
-                                                                  const PackedRates pr) {
+__global__ void __launch_bounds__(128, (kStep2Blocks<T, kWalls>))
+    step2_kernel(const StepIO<T> io, const StepArgs a, const PackedRates pr) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
     if (2 * t >= row_end<T, kRag>(a.g.nx) || y >= a.g.ny) return;
@@ -820,15 +819,19 @@ __global__ void __launch_bounds__(128, kStep2Blocks<T>) step2_kernel(const StepI
 // kForce = false (no force anywhere) compiles the force-free cascade alone:
 // without the forced path beside it the kernel needs fewer registers (no
 // spills at 5 blocks per SM with 16-bit storage, against 104-128 bytes;
-// FP16 77.2k against 70.7k MLUPS at 256^3).  Blocks per SM with 16-bit
-// storage, from measurement: 6 without force (32-56 bytes of spills; FP16
-// 79.2k MLUPS, 78.2k at 7), 5 with it; FP32 storage 4 (no spills; without
-// force its 94 registers admit 5).
-template <typename T, bool kForce>
-constexpr int kQ15Blocks = Storage<T>::kScaled ? (kForce ? 5 : 6) : 4;
+// FP16 77.2k against 70.7k MLUPS at 256^3).  Blocks per SM, by measurement at
+// 256^3 (us a step): 16-bit 6 without force (BF16 220 / 222 / 227 at 6 / 5 / 7,
+// walled FP16 198 / 212 / 204), FP16 without walls 7 (196.6 / 201.7 at 7 / 6; in
+// ragged rows 53.3 / 51.2 at 250 x 128 x 128), 5 with it (FP16 245 / 262 / 257 at
+// 5 / 4 / 6); FP32 storage 4 (no spills; without force its 94 registers admit 5).
+template <typename T, bool kWalls, bool kForce, bool kRag>
+constexpr int kQ15Blocks = !Storage<T>::kScaled                           ? 4
+                           : kForce                                       ? 5
+                           : kWalls || kRag || Storage<T>::kRef           ? 6
+                                                                          : 7;
 
 template <typename T, bool kWalls, bool kForce, bool kRag, bool kShort = false>
-__global__ void __launch_bounds__(128, (kQ15Blocks<T, kForce>))
+__global__ void __launch_bounds__(128, (kQ15Blocks<T, kWalls, kForce, kRag>))
     step2_q15_kernel(const StepIO<T> io, const StepArgs a, const PackedRates pr) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
