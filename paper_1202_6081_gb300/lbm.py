@@ -51,6 +51,8 @@ class LBMError(RuntimeError):
 def load():
     """Load liblbm.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -119,20 +121,25 @@ def _check(status, where, ctx=None):
         raise LBMError(status, where, detail)
 
 
+# The small calls (a force and one step at a time, the adjoint steps of a small
+# grid) take as long as their marshalling: array types made once, addresses as
+# plain integers (the argument types turn them into pointers), and the current
+# stream's handle without a Stream object around it.
+_ARRAY = {n: ctypes.c_double * n for n in (3, 15, 27)}
+
+
 def _darr(values, n):
-    arr = (ctypes.c_double * n)(*[float(v) for v in values])
-    return arr
+    return (_ARRAY.get(n) or ctypes.c_double * n)(*map(float, values))
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 # ---- C-ABI functions (same names, same argument order) --------------------
