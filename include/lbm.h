@@ -302,7 +302,7 @@ lbm_status lbm_macroscopic_seed(lbm_ctx *ctx, const void *f, const float *g_rho,
  *        sum_x (rho - 1), then sum_x rho u_x, rho u_y, rho u_z.  Note: the
  *        first value is the mass minus the cell count nx*ny*nz (the FP64
  *        sum of the density deviations, without the large constant).
- * Limit: ny * nz <= 65536 (one partial record per (y, z) row); larger grids
+ * Limit: ny * nz <= 65536 (at most one partial record per (y, z) row); larger grids
  * return LBM_EINVAL.  The context's device must be current (LBM_ESTATE
  * otherwise).  The first call on a device looks up the array's device
  * address (cudaGetSymbolAddress) and keeps it for the life of the process;

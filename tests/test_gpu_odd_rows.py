@@ -74,3 +74,19 @@ def test_results_do_not_depend_on_the_padding(lbm, Q, storage, n):
         out.append(S.get_state().cpu().numpy())
     assert np.isfinite(out[0]).all()
     np.testing.assert_array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("Q", [27, 15])
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("walls", [0, 3])
+@pytest.mark.parametrize("n", [2, 30, 34, 72, 130, 258, 384])
+def test_ragged_rows_in_place_equal_two_buffers_bitwise(lbm, Q, storage, walls, n):
+    shape = (4, 5, n)
+    states = []
+    for inplace in (False, True):
+        S = lbm.Solver(Q, shape, _rates(Q, False), walls=walls, force=(1e-4, -1e-4, 0),
+                       storage=storage, inplace=inplace)
+        S.set_state(W.random_field_state(shape, Q, spread=0.2))
+        S.step(5)
+        states.append(S.get_state())
+    assert torch.equal(*states)
