@@ -659,15 +659,19 @@ __global__ void __launch_bounds__(128) step1_kernel(const StepIO<float> io, cons
     float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f, ux, uy, uz;
     if (Q == 27 || kForm) cell_force(a, dense_index(a.g, x, y, z), N, Fx, Fy, Fz);
     const typename Rates<Q>::type r = load_rates<Q>(a);
-    if constexpr (Q == 27)
-        // periodic, the general form schedules better (9^3: 2.20 / 2.39 us; walled
-        // 2.65 / 2.27)
-        collide27_g<float, false, kForm && kWalls>(f, Fx, Fy, Fz, r, ux, uy, uz);
+    // the rate-1 form between walls only: periodic, the general one schedules better
+    // (9^3: 2.20 / 2.39 us; walled 2.59 / 2.27)
+    constexpr bool kRateOne = Q == 27 && kForm && kWalls;
+    if constexpr (kRateOne)
+        collide27_g<float, false, true>(f, Fx, Fy, Fz, r, ux, uy, uz);
+    else if constexpr (Q == 27)
+        collide27<float>(f, Fx, Fy, Fz, r, ux, uy, uz);
     else
         collide15<float>(f, Fx, Fy, Fz, r, kForm, ux, uy, uz);
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
-        __stcs(element<false>(io.out[q], R.own + x), f[q] * store_scale<Q, float>(q));
+        constexpr float scale = kRateOne ? store_scale<Q, float>(q) : 1.0f;
+        __stcs(element<false>(io.out[q], R.own + x), scale == 1.0f ? f[q] : f[q] * scale);
     });
 }
 
