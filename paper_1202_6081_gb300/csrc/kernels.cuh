@@ -360,21 +360,47 @@ __host__ __device__ constexpr int stored_row(int nx) {
 // (at >= nx) repeat the last pair.  In a row of odd length the last pair is one
 // cell: its high lane reads in-range elements, is set to the low lane once the
 // values are in registers (even_lanes) and stored in the row's padding.
-template <bool kRag>
+// kApart (the in-place kernels, nx even): a thread past the end takes its two
+// elements of the padding as a periodic row of their own, so that it reads and
+// writes what no other thread does; the last pair's elements are overwritten by
+// that pair's thread meanwhile.
+template <bool kRag, bool kApart = false>
 struct PairCols {
     int at, x0, xm, xp, nx;
-    __device__ __forceinline__ PairCols(int x, int n) : at(x), x0(x), nx(n) {
-        if (kRag) x0 = min(x0, (nx - 1) & ~1);
+    __host__ __device__ __forceinline__ PairCols(int x, int n) : at(x), x0(x), nx(n) {
+        if (kRag && !kApart) x0 = last_pair();
         xm = (x0 == 0) ? nx - 1 : x0 - 1;
         xp = (kRag ? x0 + 2 >= nx : x0 + 2 == nx) ? 0 : x0 + 2;
+        if (kRag && kApart && at >= nx) {
+            xm = at + 1;
+            xp = at;
+        }
     }
-    __device__ __forceinline__ bool single() const { return kRag && x0 + 1 == nx; }
-    __device__ __forceinline__ int x1() const { return single() ? 0 : x0 + 1; }
+    __host__ __device__ __forceinline__ bool single() const { return kRag && x0 + 1 == nx; }
+    __host__ __device__ __forceinline__ int x1() const { return single() ? 0 : x0 + 1; }
+    // the pair's column in a dense field, which has no padding
+    __host__ __device__ __forceinline__ int field() const {
+        return kRag && kApart ? last_pair() : x0;
+    }
+    // The same columns, in ragged rows from a value that the compiler cannot trace:
+    // it would keep the addresses of the loads for the stores, and spill
+    // (aa_odd_kernel D3Q27, periodic: 28-120 bytes, against none).
+    __device__ __forceinline__ PairCols again() const {
+        if constexpr (!kRag) return *this;
+        int x = at;
+        asm volatile("" : "+r"(x));
+        return PairCols(x, nx);
+    }
+
+private:
+    __host__ __device__ __forceinline__ int last_pair() const {
+        return min(at, (nx - 1) & ~1);
+    }
 };
 
 // End of the cells a row's threads store (T: the type stored).
 template <typename T, bool kRag>
-__device__ __forceinline__ int row_end(int nx) {
+__host__ __device__ __forceinline__ int row_end(int nx) {
     return kRag ? stored_row<T>(nx) : nx;
 }
 
@@ -416,9 +442,9 @@ __device__ __forceinline__ float4 load_ref(const float4 *p) {
 }
 
 // kSel: with the wall selects.
-template <int Q, bool kSel, bool kWalls, bool kRag>
+template <int Q, bool kSel, bool kWalls, bool kRag, bool kApart>
 __device__ __forceinline__ void add_refs_pair(const float4 *__restrict__ ref, const Rows<kWalls> &R,
-                                              const PairCols<kRag> &X, f2 (&f)[Q]) {
+                                              const PairCols<kRag, kApart> &X, f2 (&f)[Q]) {
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         if constexpr (has_ref<Q>(q)) {
@@ -701,8 +727,9 @@ __global__ void __launch_bounds__(128) step_sr32_kernel(const StepIO<float> io, 
 
 // The values of a plane's row (offset of its start) at x0 - i and x0 + 1 - i.
 // kRowFirst: the row's pointer, then the column (see kAAPlain).
-template <bool kPlain = false, bool kRowFirst = false, typename T, bool kRag>
-__device__ __forceinline__ f2 ld_shifted(const T *plane, int row, int i, const PairCols<kRag> &X) {
+template <bool kPlain = false, bool kRowFirst = false, typename T, bool kRag, bool kApart>
+__device__ __forceinline__ f2 ld_shifted(const T *plane, int row, int i,
+                                         const PairCols<kRag, kApart> &X) {
     if constexpr (kRowFirst) {
         plane += row;
         row = 0;
@@ -759,12 +786,12 @@ __device__ __forceinline__ void pull_pairs(const StepIO<T> &io, const Rows<kWall
 
 // Body force of the pair (x0, x0 + 1): the field (4-byte alignment only is
 // required of it: single loads), else the uniform force.
-template <bool kRag = false>
-__device__ __forceinline__ void pair_force(const StepArgs &a, const PairCols<kRag> &X, int y, int z,
-                                           f2 &Fx, f2 &Fy, f2 &Fz) {
+template <bool kRag, bool kApart>
+__device__ __forceinline__ void pair_force(const StepArgs &a, const PairCols<kRag, kApart> &X,
+                                           int y, int z, f2 &Fx, f2 &Fy, f2 &Fz) {
     if (a.Ffield) {
         const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
-        const float *p = a.Ffield + dense_index(a.g, X.x0, y, z);
+        const float *p = a.Ffield + dense_index(a.g, X.field(), y, z);
         const int n = X.single() ? 0 : 1;
         Fx = f2(__ldg(p), __ldg(p + n));
         Fy = f2(__ldg(p + N), __ldg(p + N + n));
@@ -917,7 +944,7 @@ struct PairCollide<15> {
 // producers are the pull sources, see lattice.cuh), then the load scale.
 template <int Q, typename T, bool kWalls, bool kRag>
 __device__ __forceinline__ void pair_inputs(const StepIO<T> &io, const Rows<kWalls> &R,
-                                            const PairCols<kRag> &X, f2 (&f)[Q]) {
+                                            const PairCols<kRag, true> &X, f2 (&f)[Q]) {
     if constexpr (Storage<T>::kRef) add_refs_pair<Q, kWalls>(io.ref_in, R, X, f);
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
@@ -930,17 +957,15 @@ __device__ __forceinline__ void pair_inputs(const StepIO<T> &io, const Rows<kWal
 template <int Q, typename T, bool kEq, bool kForce, bool kRag>
 __device__ __forceinline__ float4 pair_collide(const StepIO<T> &io, const StepArgs &a,
                                                const PackedRates &pr,
-                                               const PairCols<kRag> &X, int y, int z, int own,
-                                               f2 (&f)[Q]) {
+                                               const PairCols<kRag, true> &X, int y, int z,
+                                               int own, f2 (&f)[Q]) {
     f2 Fx = f2(0.0f), Fy = f2(0.0f), Fz = f2(0.0f), ux, uy, uz;
     if constexpr (kForce) pair_force(a, X, y, z, Fx, Fy, Fz);
     PairCollide<Q>::template run<kFoldedLoad<Q, T>(), kEq, kForce>(f, Fx, Fy, Fz, pr, ux, uy, uz);
     float4 J = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if constexpr (Storage<T>::kRef) {
         J = pair_ref(ux, uy, uz);
-        // where the thread stores: past the row's end that is the padding's, not
-        // the last pair's, whose slots its own thread may have overwritten by now
-        __stcs(io.ref_out + ((own - X.x0 + X.at) >> 1), J);
+        __stcs(io.ref_out + (own >> 1), J);
     }
     return J;
 }
@@ -960,10 +985,9 @@ __global__ void __launch_bounds__(128) aa_even_kernel(const StepIO<T> io, const 
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
     if (2 * t >= row_end<T, kRag>(a.g.nx) || y >= a.g.ny) return;
-    const PairCols<kRag> X(2 * t, a.g.nx);
-    const int x0 = X.x0;
+    const PairCols<kRag, true> X(2 * t, a.g.nx);
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);  // producers of the values (BF16)
-    const int own = R.own + x0;
+    const int own = R.own + X.at;
     f2 f[Q];
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
@@ -977,8 +1001,7 @@ __global__ void __launch_bounds__(128) aa_even_kernel(const StepIO<T> io, const 
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         const f2 v = stored_pair<Q, T, q>(f[q], store_scale<Q, T>(q), J);
-        Pair<T>::template st2s<q>(element<kRag, kPlain>(io.out[opposite<Q>(q)], R.own + X.at), v,
-                                  seed);
+        Pair<T>::template st2s<q>(element<kRag, kPlain>(io.out[opposite<Q>(q)], own), v, seed);
     });
 }
 
@@ -996,11 +1019,9 @@ __global__ void __launch_bounds__(128, (kAAOddBlocks<Q, T, kForce>))
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
     if (2 * t >= row_end<T, kRag>(a.g.nx) || y >= a.g.ny) return;
-    const PairCols<kRag> X(2 * t, a.g.nx);
-    const int x0 = X.x0, xm = X.xm, xp = X.xp;
-    const bool past = kRag && X.at != x0;
+    const PairCols<kRag, true> X(2 * t, a.g.nx);
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
-    const int own = R.own + x0;
+    const int own = R.own + X.at;
     // rows along a wall take the wall selects, the others the plain accesses
     // (see pull_pairs)
     const bool edge = kWalls && (R.edge || blockDim.x < 32);
@@ -1025,6 +1046,7 @@ __global__ void __launch_bounds__(128, (kAAOddBlocks<Q, T, kForce>))
     if constexpr (!kSeedAfterCollision<Q, T>) seed = pair_seed<Q>(f, own);
     const float4 J = pair_collide<Q, T, kEq, kForce>(io, a, pr, X, y, z, own, f);
     if constexpr (kSeedAfterCollision<Q, T>) seed = pair_seed<Q>(f, own);
+    const PairCols<kRag, true> Y = X.again();
     const auto store = [&](auto sel) {
         static_for<Q>([&](auto iq) {
             constexpr int q = decltype(iq)::value;
@@ -1033,18 +1055,16 @@ __global__ void __launch_bounds__(128, (kAAOddBlocks<Q, T, kForce>))
             const f2 v = stored_pair<Q, T, q>(f[q], store_scale<Q, T>(q), J);
             // downstream neighbour x + e_q: the row of the mirrored pull
             if (decltype(sel)::value && R.wall[2 - j][2 - k]) {
-                Pair<T>::template st2s<q>(element<kRag, kPlain>(io.out[o], R.own + X.at), v, seed);
+                Pair<T>::template st2s<q>(element<kRag, kPlain>(io.out[o], own), v, seed);
             } else {
                 const int row = R.off[2 - j][2 - k];
                 const auto dst = [&](int x) { return element<kRag, kPlain>(io.out[q], row + x); };
                 if constexpr (i == 0)
-                    Pair<T>::template st2s<q>(dst(X.at), v, seed);
+                    Pair<T>::template st2s<q>(dst(Y.x0), v, seed);
                 else if constexpr (i == 1)
-                    Pair<T>::template st1x2s<q>(dst(past ? X.at : x0 + 1),
-                                                dst(past ? X.at + 1 : xp), v, seed);
+                    Pair<T>::template st1x2s<q>(dst(Y.x0 + 1), dst(Y.xp), v, seed);
                 else
-                    Pair<T>::template st1x2s<q>(dst(past ? X.at : xm), dst(past ? X.at + 1 : x0),
-                                                v, seed);
+                    Pair<T>::template st1x2s<q>(dst(Y.xm), dst(Y.x0), v, seed);
             }
         });
     };

@@ -1,0 +1,62 @@
+// Host program over the kernels' index arithmetic (no GPU, no kernel launched):
+// prints "ok" or the first thing that is wrong.
+#include <cstdio>
+#include <cstdlib>
+#include <vector>
+
+#include "kernels.cuh"
+
+#define REQUIRE(c, ...)                    \
+    do {                                   \
+        if (!(c)) {                        \
+            std::printf("wrong: %s ", #c); \
+            std::printf(__VA_ARGS__);      \
+            std::printf("\n");             \
+            std::exit(1);                  \
+        }                                  \
+    } while (0)
+
+// An in-place step of a ragged row of nx cells.  A plane is read by the
+// population opposite to the one that writes it: where the writer stores columns
+// (x0 + i, x0 + 1 + i), the reader, moving by -i, loads the same.  Every element
+// up to the end of the last sector belongs to one thread: no other one reads it
+// or writes it.
+template <typename T>
+void in_place_row(int nx) {
+    const int end = lbm::row_end<T, true>(nx);
+    for (int i = -1; i <= 1; ++i) {
+        std::vector<int> reader(end, -1), writer(end, -1);
+        const auto claim = [&](std::vector<int> &who, int x, int t) {
+            REQUIRE(x >= 0 && x < end, "nx %d shift %d thread %d column %d", nx, i, t, x);
+            REQUIRE(who[x] < 0, "nx %d shift %d column %d threads %d, %d", nx, i, x, who[x], t);
+            who[x] = t;
+        };
+        for (int t = 0; 2 * t < end; ++t) {
+            const lbm::PairCols<true, true> X(2 * t, nx);
+            const int store[2] = {i == 0 ? X.x0 : i == 1 ? X.x0 + 1 : X.xm,
+                                  i == 0 ? X.x0 + 1 : i == 1 ? X.xp : X.x0};
+            const int load[2] = {i == 0 ? X.x0 : i == 1 ? X.x1() : X.xm,
+                                 i == 0 ? X.x0 + 1 : i == 1 ? X.xp : X.x0};
+            for (int k = 0; k < 2; ++k) {
+                claim(writer, store[k], t);
+                claim(reader, load[k], t);
+                if (X.at < nx)  // a cell: the periodic row
+                    REQUIRE(store[k] == (X.at + k + i + nx) % nx, "nx %d shift %d thread %d", nx, i,
+                            t);
+            }
+            REQUIRE(X.x0 == X.at && !X.single(), "nx %d thread %d", nx, t);
+            REQUIRE(X.field() + 1 < nx && (X.at >= nx || X.field() == X.at), "nx %d thread %d", nx,
+                    t);
+        }
+        REQUIRE(reader == writer, "nx %d shift %d", nx, i);
+    }
+}
+
+int main() {
+    for (int nx = 2; nx <= 600; nx += 2) {
+        in_place_row<float>(nx);
+        in_place_row<__half>(nx);
+    }
+    std::printf("ok\n");
+    return 0;
+}
