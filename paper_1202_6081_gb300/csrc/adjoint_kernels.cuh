@@ -117,9 +117,10 @@ __global__ void __launch_bounds__(128, (kAdjointBlocks<T, kRag, kEq>)) adjoint2_
     f2 Fx, Fy, Fz;
     pair_force(a, X, y, z, Fx, Fy, Fz);
     // the dJ/dF accumulator is read now, so its latency hides behind the
-    // collision's reverse; it is written back at the end
+    // collision's reverse; it is written back at the end.  A thread that repeats
+    // the last pair leaves it to that pair's own thread, which overwrites it.
     f2 acc[3] = {f2(0.0f), f2(0.0f), f2(0.0f)};
-    if (g.gF) {
+    if (g.gF && X.owner()) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const float *p = g.gF + d * N + c;
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(128, (kAdjointBlocks<T, kRag, kEq>)) adjoint2_
         constexpr int q = decltype(iq)::value;
         Pair<float>::st2(element<kRag>(g.lam_out[q], R.own + X.at), lam[q]);
     });
-    if (g.gF && (!kRag || X.at == X.x0)) {
+    if (g.gF && X.owner()) {
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             float *p = g.gF + d * N + c;

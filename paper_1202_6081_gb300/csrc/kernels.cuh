@@ -378,6 +378,8 @@ struct PairCols {
     }
     __host__ __device__ __forceinline__ bool single() const { return kRag && x0 + 1 == nx; }
     __host__ __device__ __forceinline__ int x1() const { return single() ? 0 : x0 + 1; }
+    // whether the pair's cells are this thread's
+    __host__ __device__ __forceinline__ bool owner() const { return !kRag || at < nx; }
     // the pair's column in a dense field, which has no padding
     __host__ __device__ __forceinline__ int field() const {
         return kRag && kApart ? last_pair() : x0;

@@ -52,7 +52,32 @@ void in_place_row(int nx) {
     }
 }
 
+// A two-buffer step, and an adjoint step with its accumulator (a dense field,
+// read and written in place): every cell of the field has one owner.
+template <typename T>
+void two_buffer_row(int nx) {
+    const int end = lbm::row_end<T, true>(nx);
+    std::vector<int> owner(nx, -1);
+    for (int t = 0; 2 * t < end; ++t) {
+        const lbm::PairCols<true> X(2 * t, nx);
+        REQUIRE(X.field() == X.x0 && X.x0 >= 0 && X.x0 < nx, "nx %d thread %d", nx, t);
+        REQUIRE(X.xm == (X.x0 + nx - 1) % nx && X.xp == (X.single() ? 0 : (X.x0 + 2) % nx) &&
+                    X.x1() == (X.x0 + 1) % nx,
+                "nx %d thread %d", nx, t);
+        if (!X.owner()) continue;
+        for (int x = X.x0; x < X.x0 + (X.single() ? 1 : 2); ++x) {
+            REQUIRE(x < nx && owner[x] < 0, "nx %d column %d thread %d", nx, x, t);
+            owner[x] = t;
+        }
+    }
+    for (int x = 0; x < nx; ++x) REQUIRE(owner[x] == x / 2, "nx %d column %d", nx, x);
+}
+
 int main() {
+    for (int nx = 1; nx <= 600; ++nx) {
+        two_buffer_row<float>(nx);
+        two_buffer_row<__half>(nx);
+    }
     for (int nx = 2; nx <= 600; nx += 2) {
         in_place_row<float>(nx);
         in_place_row<__half>(nx);
