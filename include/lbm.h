@@ -150,7 +150,9 @@ void lbm_destroy(lbm_ctx *ctx);
  * 32 elements), in the storage type; for LBM_STORE_BF16 followed by the
  * momentum references (one float4 per pair of cells of the pitched rows,
  * 8 bytes per cell; two such arrays with LBM_INPLACE).  A state is fully
- * described by these bytes: copying them copies the state.  0 for a NULL
+ * described by these bytes: copying them copies the state.  The elements of a
+ * row past nx are the library's: steps store whole 32-byte sectors and write
+ * some of them, and no result depends on what they hold.  0 for a NULL
  * context. */
 size_t lbm_state_bytes(const lbm_ctx *ctx);
 
@@ -254,7 +256,9 @@ lbm_status lbm_step_into(lbm_ctx *ctx, const void *f_in, void *f_out, void *stre
  * (device FP32 [3][nz][ny][nx], accumulated; the force of step t is the
  * bound force field or the uniform force).  lam_next, lam_out: device FP32
  * adjoint fields (lbm_adjoint_bytes, 16-byte aligned, not overlapping: the
- * step reads lam_next at neighbouring cells while it writes lam_out).
+ * step reads lam_next at neighbouring cells while it writes lam_out).  In the
+ * padding of lam_out's rows the step leaves what is there or stores zeros, so
+ * sums over a whole field of zero padding are sums over its cells.
  * Errors: LBM_EINVAL, LBM_EUNSUPPORTED (LBM_INPLACE context), LBM_ECUDA. */
 lbm_status lbm_adjoint_step(lbm_ctx *ctx, const void *f_t, const float *lam_next,
                             float *lam_out, float *dJdF, void *stream);

@@ -104,7 +104,6 @@ __global__ void __launch_bounds__(128, (kAdjointBlocks<T, kRag, kEq>)) adjoint2_
         pull_adjoint<Q, kWalls>(g, R, X, mu);
     else
         pull_adjoint<Q, false>(g, R, X, mu);
-    even_lanes(X, mu);
     // deviations f - w: 16-bit values scaled by w
     if constexpr (Storage<T>::kScaled) {
         static_for<Q>([&](auto iq) {
@@ -130,6 +129,7 @@ __global__ void __launch_bounds__(128, (kAdjointBlocks<T, kRag, kEq>)) adjoint2_
     const typename PairRates<Q>::type r = PairRates<Q>::load(pr);
     f2 lam[Q], gF[3];
     adjoint_collide<kEq, f2>(f, Fx, Fy, Fz, r, mu, lam, gF[0], gF[1], gF[2]);
+    zero_padding(X, lam);
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         Pair<float>::st2(element<kRag>(g.lam_out[q], R.own + X.at), lam[q]);

@@ -416,6 +416,17 @@ __device__ __forceinline__ void even_lanes(const PairCols<kRag> &X, f2 (&f)[Q]) 
     }
 }
 
+// Zeros in the lanes that a thread stores in its row's padding.
+template <int Q, bool kRag>
+__device__ __forceinline__ void zero_padding(const PairCols<kRag> &X, f2 (&f)[Q]) {
+    if constexpr (kRag) {
+        if (X.single() || !X.owner()) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) f[q] = f2(X.owner() ? f[q].lo() : 0.0f, 0.0f);
+        }
+    }
+}
+
 // BF16 momentum references (see lattice.cuh) for the pair kernels.
 //
 // Reader: adds to the pulled raw values f[q] of cells (x0, x0 + 1) the
