@@ -1,0 +1,65 @@
+"""FP32 rows of odd length on grids above the size that the one-cell step kernel
+serves (8,192 cells, 20,480 between walls): the two-cell kernel, whose last thread
+of a row has one cell and whose threads past it store in the padding."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+SHAPES = [(9, 10, 257), (30, 31, 33)]  # 23,130 and 30,690 cells
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1202_6081_gb300 import build
+    from paper_1202_6081_gb300 import lbm as mod
+    build()
+    mod.load()
+    return mod
+
+
+def _solver(lbm, Q, shape, walls, form):
+    """form: D3Q27 the rate-1 relaxation, D3Q15 a force (a field)."""
+    om = W.omegas(Q, 1 / 0.6) if Q == 27 and form else W.random_omegas(Q, seed=12)
+    F = np.asarray(W.rng(13).uniform(-2e-3, 2e-3, (3,) + shape), dtype=np.float32)
+    if Q == 15 and not form:
+        F = np.zeros(3)
+    return lbm.Solver(Q, shape, om, walls=walls, force=F), om, F.astype(np.float64)
+
+
+@pytest.mark.parametrize("Q", [27, 15])
+@pytest.mark.parametrize("walls", [0, 3])
+@pytest.mark.parametrize("form", [False, True])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_step_matches_oracle(lbm, Q, walls, form, shape):
+    """One step against the FP64 oracle, at the bound of the other FP32 steps (from
+    this state the D3Q27 flow has no positive density after three)."""
+    import oracle
+    f = W.random_field_state(shape, Q, seed=14, spread=0.5)
+    S, om, F = _solver(lbm, Q, shape, walls, form)
+    S.set_state(f)
+    S.step(1)
+    want = oracle.run(Q, shape, f, F, om, 1, bc=walls)
+    assert np.abs(S.get_state().cpu().numpy() - want).max() <= 2e-6
+
+
+@pytest.mark.parametrize("Q", [27, 15])
+@pytest.mark.parametrize("walls", [0, 3])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_results_do_not_depend_on_the_padding(lbm, Q, walls, shape):
+    out = []
+    for fill in (0x00, 0xff):  # zeros, NaNs
+        S = _solver(lbm, Q, shape, walls, True)[0]
+        for b in S.buffers:
+            b.fill_(fill)
+        S.set_state(W.random_field_state(shape, Q, spread=0.2))
+        S.step(5)
+        out.append(S.get_state())
+    assert torch.isfinite(out[0]).all()
+    assert torch.equal(*out)
