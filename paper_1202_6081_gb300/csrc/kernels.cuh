@@ -162,7 +162,7 @@ struct StepIO {
 // 16-bit D3Q27 step (256^3: FP16 327 against 338 us, BF16 391 against 398), whose
 // registers are short, and some in-place kernels (kAAPlain).
 template <bool kRag, bool kPlain = false, typename T>
-__device__ __forceinline__ T *element(T *plane, int e) {
+__host__ __device__ __forceinline__ T *element(T *plane, int e) {
     using Byte = typename std::conditional<std::is_const<T>::value, const char, char>::type;
     if constexpr (kPlain || (kRag && sizeof(T) == 4))
         return plane + e;

@@ -73,7 +73,37 @@ void two_buffer_row(int nx) {
     for (int x = 0; x < nx; ++x) REQUIRE(owner[x] == x / 2, "nx %d column %d", nx, x);
 }
 
+// The last element of a plane, in the form that the dispatch gives the grid
+// (ragged()): byte offsets wrap at 2^32.  No memory is touched.
+template <typename T>
+void last_element(int nx, int ny, int nz, bool want) {
+    lbm::Grid g{};
+    g.nx = nx;
+    g.ny = ny;
+    g.nz = nz;
+    g.px = (nx + 31) / 32 * 32;
+    g.pop = (long long)g.px * ny * nz;
+    const bool rag = lbm::ragged<T>(g);
+    REQUIRE(rag == want, "%d x %d x %d of %d bytes", nx, ny, nz, int(sizeof(T)));
+    T *const plane = reinterpret_cast<T *>(uintptr_t(1) << 40);
+    const int e = int(g.pop - 1);
+    const T *const at[2] = {rag ? lbm::element<true>(plane, e) : lbm::element<false>(plane, e),
+                            rag ? lbm::element<true, true>(plane, e)
+                                : lbm::element<false, true>(plane, e)};
+    for (const T *p : at)
+        REQUIRE(reinterpret_cast<uintptr_t>(p) ==
+                    reinterpret_cast<uintptr_t>(plane) + uintptr_t(e) * sizeof(T),
+                "%d x %d x %d of %d bytes", nx, ny, nz, int(sizeof(T)));
+}
+
 int main() {
+    last_element<float>(1024, 1024, 1024, false);  // 2^32 bytes
+    last_element<float>(1024, 1024, 1025, true);
+    last_element<float>(32, 32768, 1025, true);
+    last_element<float>(1536, 1024, 1024, true);
+    last_element<float>(1023, 1024, 1024, true);  // ragged by its rows
+    last_element<__half>(1024, 1024, 2047, false);
+    last_element<__half>(1022, 1024, 2047, true);
     for (int nx = 1; nx <= 600; ++nx) {
         two_buffer_row<float>(nx);
         two_buffer_row<__half>(nx);
