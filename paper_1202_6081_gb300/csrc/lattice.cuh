@@ -1,5 +1,5 @@
-// Lattice constants, state storage and the pull-streaming gather shared by
-// the kernels of liblbm.so.
+// Lattice constants, state storage and layout shared by the kernels of
+// liblbm.so.
 //
 // State layout in HBM: structure of arrays, population-major,
 //   buf[alpha][z][y][x_pitched],  alpha in the paper's velocity order,
@@ -104,7 +104,6 @@ template <>
 struct Storage<float> {
     static constexpr bool kScaled = false;
     static constexpr bool kRef = false;
-    __device__ __forceinline__ static float load(const float *p) { return __ldg(p); }
     __device__ __forceinline__ static void store(float *p, float v) { __stcs(p, v); }
 };
 
@@ -112,9 +111,6 @@ template <>
 struct Storage<__half> {
     static constexpr bool kScaled = true;
     static constexpr bool kRef = false;
-    __device__ __forceinline__ static float load(const __half *p) {
-        return __half2float(__ldg(p));
-    }
     __device__ __forceinline__ static void store(__half *p, float v) {
         __stcs(reinterpret_cast<unsigned short *>(p), __half_as_ushort(__float2half_rn(v)));
     }
@@ -124,9 +120,6 @@ template <>
 struct Storage<__nv_bfloat16> {
     static constexpr bool kScaled = true;
     static constexpr bool kRef = true;  // momentum references, see below
-    __device__ __forceinline__ static float load(const __nv_bfloat16 *p) {
-        return __bfloat162float(__ldg(p));
-    }
     __device__ __forceinline__ static void store(__nv_bfloat16 *p, float v) {
         __stcs(reinterpret_cast<unsigned short *>(p),
                __bfloat16_as_ushort(__float2bfloat16_rn(v)));
@@ -244,7 +237,6 @@ struct Grid {
     int nx, ny, nz;   // cells
     int px;           // row pitch in elements
     unsigned bc;      // kWallY | kWallZ
-    long long plane;  // px * ny
     long long pop;    // px * ny * nz: distance between populations
     int layout;       // kPull, kAANatural or kAASwapped (state reads and writes)
 };
