@@ -250,6 +250,7 @@ lbm_status lbm_create(lbm_lattice lattice, int nx, int ny, int nz, const double 
     c->g.layout = inplace ? lbm::kAANatural : lbm::kPull;
     c->inplace = inplace;
     c->sr32 = sr32;
+    c->g.plane = px * ny;
     c->g.pop = px * ny * nz;
     for (int b = 0; b < 27; ++b) c->w[b] = (b >= 4 && b < Q) ? float(omega[b]) : 0.0f;
     for (int i = 0; i < 3; ++i) c->F[i] = force ? float(force[i]) : 0.0f;
