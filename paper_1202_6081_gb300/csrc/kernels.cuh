@@ -21,9 +21,16 @@ struct StepArgs {
     int sr32;              // FP32 storage: incremental update, stochastically rounded
 };
 
+constexpr int kSMs = 152;
+
 // Launch geometry shared by the per-cell kernels (cell_launch below).
 struct CellLaunch {
     dim3 grid, block;
+    // warps of the SM with the most blocks
+    int sm_warps() const {
+        const long long blocks = (long long)grid.x * grid.y * grid.z;
+        return int((blocks + kSMs - 1) / kSMs * ((block.x * block.y + 31) / 32));
+    }
 };
 
 // Blocks of at most 128 threads along x: rows of at least 17 threads take whole
@@ -686,7 +693,7 @@ __device__ __forceinline__ void pull_cell(const StepIO<float> &io, const Rows<kW
 // one thread's chain of instructions, which is shorter here.  (Scalar
 // arithmetic rounds differently from the packed one, so grids that can also run
 // in place, with even rows, keep the two-cell kernel at every size: their
-// states are the same bit for bit in either scheme.)  See kSmallCells.
+// states are the same bit for bit in either scheme.)  See kOneCellWarps.
 template <int Q, bool kWalls, bool kForm>
 __global__ void __launch_bounds__(128) step1_kernel(const StepIO<float> io, const StepArgs a) {
     int x, y, z;
@@ -1221,7 +1228,7 @@ __global__ void __launch_bounds__(128) macro_kernel(const StepIO<T> io, const St
 // are FP32 sums of its stored deviations; the running sums across cells are
 // FP64.
 constexpr int kFinalThreads = 256;
-constexpr int kRedBlocks = 152 * 8;
+constexpr int kRedBlocks = kSMs * 8;
 
 struct RedLaunch {
     dim3 block;
@@ -1361,21 +1368,24 @@ bool ragged(const Grid &g) {
     return stored_row<T>(g.nx) != g.nx || g.pop * (long long)sizeof(T) > (1ll << 32);
 }
 
-// FP32 grids of odd rows up to this many cells take the one-cell step kernel.
-// us a step, one cell / two cells per thread / one-cell kernel before this one:
-// D3Q27 periodic 9^3 2.27 / 2.19 / 2.26, 17^3 2.33 / 2.51 / 2.20, 25^3 2.78 /
-// 2.64 / 2.82, 33^3 3.16 / 3.10 / 3.48; walled 9^3 2.26 / 2.78 / 2.57, 3 x 43 x 43
-// 2.78 / 3.74 / 3.03, 25^3 2.78 / 3.44 / 3.06, 33^3 3.80 / 3.22 / 3.99.
-constexpr long long kSmallCells = 8192, kSmallWalledCells = 20480;
+// Grids of odd rows take the one-cell step kernel where its launch leaves no SM
+// more than this many warps: a step is one thread's chain of instructions there.
+// us a step, one cell / two cells per thread, FP32, warps in brackets: D3Q27
+// periodic 23^3 (4) 2.25 / 2.57, 257 x 10 x 9 (6) 2.44 / 2.82, 25^3 (8) 2.72 / 2.63;
+// walled 23^3 2.31 / 3.21, 27^3 (8) 2.82 / 3.29, 33^3 (16) 3.79 / 3.27; D3Q15
+// periodic with force 23^3 1.87 / 2.31, walled 23^3 2.06 / 2.25, 27^3 2.36 / 2.32,
+// without force 2.06 / 2.12.  Rows of one cell take the two-cell kernel (1 x 100 x
+// 100 walled 6.94 / 5.39).
+template <int Q, typename T, bool kWalls>
+constexpr int kOneCellWarps = !std::is_same<T, float>::value ? 0 : kWalls || Q == 15 ? 8 : 6;
 
 // kForm: the rate-1 relaxation (D3Q27), a force anywhere (D3Q15).
 template <int Q, typename T, bool kWalls, bool kForm>
 void launch_step_kernel(const StepIO<T> &io, const StepArgs &a, const PackedRates &pr,
                       cudaStream_t st) {
-    if constexpr (std::is_same<T, float>::value) {
-        const long long cells = (long long)a.g.nx * a.g.ny * a.g.nz;
-        if (a.g.nx % 2 && cells <= (kWalls ? kSmallWalledCells : kSmallCells)) {
-            const CellLaunch L = cell_launch(a.g);
+    if constexpr (kOneCellWarps<Q, T, kWalls> > 0) {
+        const CellLaunch L = cell_launch(a.g);
+        if (a.g.nx % 2 && a.g.nx > 1 && L.sm_warps() <= kOneCellWarps<Q, T, kWalls>) {
             step1_kernel<Q, kWalls, kForm><<<L.grid, L.block, 0, st>>>(io, a);
             return;
         }

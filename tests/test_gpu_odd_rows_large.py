@@ -1,6 +1,6 @@
-"""FP32 rows of odd length on grids above the size that the one-cell step kernel
-serves (8,192 cells, 20,480 between walls): the two-cell kernel, whose last thread
-of a row has one cell and whose threads past it store in the padding."""
+"""Rows of odd length on grids above the size that the one-cell kernels serve (16
+warps on an SM): the two-cell kernels, whose last thread of a row has one cell and
+whose threads past it store in the padding."""
 import numpy as np
 import pytest
 
@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-SHAPES = [(9, 10, 257), (30, 31, 33)]  # 23,130 and 30,690 cells
+SHAPES = [(20, 21, 257), (30, 41, 41)]  # 27 and 20 warps
 
 
 @pytest.fixture(scope="module")
