@@ -515,12 +515,11 @@ __device__ __forceinline__ f2 stored_pair(f2 v, float sc, const float4 &J) {
 // population (as in the step kernels), and the common case -- two-buffer
 // layout, no walls -- without the layout and wall selects.
 
-// Population q's stored value at plane + src -> deviation f - w; prod: the cell
-// whose collision produced it (the momentum reference of BF16 storage).
+// Population q's stored value -> deviation f - w; prod: the cell whose collision
+// produced it (the momentum reference of BF16 storage).
 template <int Q, typename T, int q>
-__device__ __forceinline__ float load_cell(const T *plane, int src, const float4 *ref, int prod,
-                                           bool wall) {
-    float v = Pair<T>::ld1(plane + src);
+__device__ __forceinline__ float load_cell(const T *at, const float4 *ref, int prod, bool wall) {
+    float v = Pair<T>::ld1(at);
     if constexpr (Storage<T>::kRef && has_ref<Q>(q)) {
         const float r = ref_dot<Q, q>(load_ref<ey<Q>(q), ez<Q>(q)>(ref + (prod >> 1)));
         v += wall ? -r : r;
@@ -538,7 +537,7 @@ __device__ __forceinline__ void gather(const StepIO<T> &io, const Grid &g, int x
         static_for<Q>([&](auto iq) {
             constexpr int q = decltype(iq)::value;
             const int src = R.off[ey<Q>(q) + 1][ez<Q>(q) + 1] + xs[ex<Q>(q) + 1];
-            f[q] = load_cell<Q, T, q>(io.in[q], src, io.ref_in, src, false);
+            f[q] = load_cell<Q, T, q>(io.in[q] + src, io.ref_in, src, false);
         });
         return;
     }
@@ -551,7 +550,7 @@ __device__ __forceinline__ void gather(const StepIO<T> &io, const Grid &g, int x
         const int prod = wall ? own : R.off[j][k] + xs[i];
         const bool opp = g.layout == kPull ? wall : g.layout == kAASwapped && !wall;
         const T *plane = opp ? io.in[opposite<Q>(q)] : io.in[q];
-        f[q] = load_cell<Q, T, q>(plane, g.layout == kAANatural ? own : prod, io.ref_in, prod,
+        f[q] = load_cell<Q, T, q>(plane + (g.layout == kAANatural ? own : prod), io.ref_in, prod,
                                   wall);
     });
 }
@@ -673,10 +672,10 @@ __device__ __forceinline__ float deviation(double f) {
     return float(f - w);
 }
 
-// One cell's pulled FP32 populations.
+// One cell's pulled populations, as deviations f - w.
 // kRag: see element().
-template <int Q, bool kRag, bool kWalls>
-__device__ __forceinline__ void pull_cell(const StepIO<float> &io, const Rows<kWalls> &R, int x,
+template <int Q, typename T, bool kRag, bool kWalls>
+__device__ __forceinline__ void pull_cell(const StepIO<T> &io, const Rows<kWalls> &R, int x,
                                           int nx, float (&f)[Q]) {
     const int xs[3] = {(x + 1 == nx) ? 0 : x + 1, x, (x == 0) ? nx - 1 : x - 1};
     static_for<Q>([&](auto iq) {
@@ -684,40 +683,74 @@ __device__ __forceinline__ void pull_cell(const StepIO<float> &io, const Rows<kW
         constexpr int i = ex<Q>(q) + 1, j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
         const bool wall = kWalls && R.wall[j][k];
         const int src = wall ? R.own + x : R.off[j][k] + xs[i];
-        f[q] = Pair<float>::ld1(element<kRag>(wall ? io.in[opposite<Q>(q)] : io.in[q], src));
+        const T *at = element<kRag>(wall ? io.in[opposite<Q>(q)] : io.in[q], src);
+        f[q] = load_cell<Q, T, q>(at, io.ref_in, src, wall);
     });
 }
 
-// One fused FP32 step, one cell per thread, for small grids with rows of odd
-// length.  A small grid does not fill the chip and its step takes as long as
+// One fused step, one cell per thread, for small grids with rows of odd length.
+// A small grid does not fill the chip and its step takes as long as
 // one thread's chain of instructions, which is shorter here.  (Scalar
 // arithmetic rounds differently from the packed one, so grids that can also run
 // in place, with even rows, keep the two-cell kernel at every size: their
 // states are the same bit for bit in either scheme.)  See kOneCellWarps.
-template <int Q, bool kWalls, bool kForm>
-__global__ void __launch_bounds__(128) step1_kernel(const StepIO<float> io, const StepArgs a) {
+// BF16 storage: the cells x (even) and x + 1, in neighbouring lanes, exchange their
+// velocities for the pair's reference, so every lane takes part: lanes beyond the
+// grid work on a clamped cell and store nothing.
+template <int Q, typename T, bool kWalls, bool kForm>
+__global__ void __launch_bounds__(128) step1_kernel(const StepIO<T> io, const StepArgs a) {
     int x, y, z;
-    if (!cell_coords(a.g, x, y, z)) return;
+    const bool inside = cell_coords(a.g, x, y, z);
+    if constexpr (Storage<T>::kRef) {
+        x = min(x, a.g.nx - 1);
+        y = min(y, a.g.ny - 1);
+    } else {
+        if (!inside) return;
+    }
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
     float f[Q];
-    pull_cell<Q, false>(io, R, x, a.g.nx, f);
+    pull_cell<Q, T, false>(io, R, x, a.g.nx, f);
+    unsigned seed = 0;
+    if constexpr (Storage<T>::kScaled) seed = cell_seed<Q>(f, R.own + x);
     const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
     float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f, ux, uy, uz;
     if (Q == 27 || kForm) cell_force(a, dense_index(a.g, x, y, z), N, Fx, Fy, Fz);
     const typename Rates<Q>::type r = load_rates<Q>(a);
     // the rate-1 form between walls only: periodic, the general one schedules better
-    // (9^3: 2.20 / 2.39 us; walled 2.59 / 2.27)
-    constexpr bool kRateOne = Q == 27 && kForm && kWalls;
+    // (9^3: 2.20 / 2.39 us; walled 2.59 / 2.27); BF16 2.76 / 3.90 at 17^3 walled
+    constexpr bool kRateOne = Q == 27 && kForm && kWalls && !Storage<T>::kRef;
     if constexpr (kRateOne)
         collide27_g<float, false, true>(f, Fx, Fy, Fz, r, ux, uy, uz);
     else if constexpr (Q == 27)
         collide27<float>(f, Fx, Fy, Fz, r, ux, uy, uz);
     else
         collide15<float>(f, Fx, Fy, Fz, r, kForm, ux, uy, uz);
+    float4 J = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if constexpr (Storage<T>::kRef) {
+        const float px = __shfl_xor_sync(0xffffffffu, ux, 1);
+        const float py = __shfl_xor_sync(0xffffffffu, uy, 1);
+        const float pz = __shfl_xor_sync(0xffffffffu, uz, 1);
+        if ((x ^ 1) < a.g.nx)  // both cells of the pair exist (a + b == b + a exactly)
+            J = make_float4(1.5f * (ux + px), 1.5f * (uy + py), 1.5f * (uz + pz), 0.0f);
+        else
+            J = make_float4(3.0f * ux, 3.0f * uy, 3.0f * uz, 0.0f);
+        J.w = J.x;
+        if (!inside) return;
+        if ((x & 1) == 0) __stcs(io.ref_out + ((R.own + x) >> 1), J);
+    }
     static_for<Q>([&](auto iq) {
         constexpr int q = decltype(iq)::value;
         constexpr float scale = kRateOne ? store_scale<Q, float>(q) : 1.0f;
-        __stcs(element<false>(io.out[q], R.own + x), scale == 1.0f ? f[q] : f[q] * scale);
+        T *at = element<false>(io.out[q], R.own + x);
+        if constexpr (Storage<T>::kScaled) {
+            float ref = 0.0f;
+            if constexpr (Storage<T>::kRef && has_ref<Q>(q)) ref = ref_dot<Q, q>(J);
+            const float v = fmaf(f[q], scale * float(1.0 / weight<Q>(q)), -ref);
+            __stcs(reinterpret_cast<unsigned short *>(at),
+                   static_cast<unsigned short>(pack_sr<T, q>(v, 0.0f, seed) & 0xffffu));
+        } else {
+            __stcs(at, scale == 1.0f ? f[q] : f[q] * scale);
+        }
     });
 }
 
@@ -731,7 +764,7 @@ __global__ void __launch_bounds__(128) step_sr32_kernel(const StepIO<float> io, 
     if (!cell_coords(a.g, x, y, z)) return;
     const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
     float f[Q];
-    pull_cell<Q, true>(io, R, x, a.g.nx, f);
+    pull_cell<Q, float, true>(io, R, x, a.g.nx, f);
     const unsigned seed = cell_seed<Q>(f, R.own + x);
     float Fx, Fy, Fz;
     const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
@@ -1376,17 +1409,25 @@ bool ragged(const Grid &g) {
 // periodic with force 23^3 1.87 / 2.31, walled 23^3 2.06 / 2.25, 27^3 2.36 / 2.32,
 // without force 2.06 / 2.12.  Rows of one cell take the two-cell kernel (1 x 100 x
 // 100 walled 6.94 / 5.39).
-template <int Q, typename T, bool kWalls>
-constexpr int kOneCellWarps = !std::is_same<T, float>::value ? 0 : kWalls || Q == 15 ? 8 : 6;
+// 16-bit storage (17^3): between walls, where the two-cell kernel's wall selects cost
+// most (D3Q27 BF16 2.8 / 5.6, at 33^3 4.8 / 5.8, FP16 2.70 / 3.53; D3Q15 BF16 2.25 /
+// 2.94, FP16 2.18 / 2.44), and D3Q27 periodic (BF16 2.31 / 3.27, FP16 at general rates
+// 2.25 / 2.70, at the rate-1 form 2.3 / 2.4 but 0.9x at 3 x 43 x 43).
+template <int Q, typename T, bool kWalls, bool kForm>
+constexpr int kOneCellWarps =
+    std::is_same<T, float>::value ? (kWalls || Q == 15 ? 8 : 6)
+    : Storage<T>::kRef            ? (kWalls ? (Q == 27 ? 16 : 12) : (Q == 27 ? 6 : 0))
+    : kWalls                      ? (Q == 27 ? 12 : 6)
+                                  : (Q == 27 && !kForm ? 6 : 0);
 
 // kForm: the rate-1 relaxation (D3Q27), a force anywhere (D3Q15).
 template <int Q, typename T, bool kWalls, bool kForm>
 void launch_step_kernel(const StepIO<T> &io, const StepArgs &a, const PackedRates &pr,
                       cudaStream_t st) {
-    if constexpr (kOneCellWarps<Q, T, kWalls> > 0) {
+    if constexpr (kOneCellWarps<Q, T, kWalls, kForm> > 0) {
         const CellLaunch L = cell_launch(a.g);
-        if (a.g.nx % 2 && a.g.nx > 1 && L.sm_warps() <= kOneCellWarps<Q, T, kWalls>) {
-            step1_kernel<Q, kWalls, kForm><<<L.grid, L.block, 0, st>>>(io, a);
+        if (a.g.nx % 2 && a.g.nx > 1 && L.sm_warps() <= kOneCellWarps<Q, T, kWalls, kForm>) {
+            step1_kernel<Q, T, kWalls, kForm><<<L.grid, L.block, 0, st>>>(io, a);
             return;
         }
     }

@@ -24,13 +24,13 @@ def lbm():
     return mod
 
 
-def _solver(lbm, Q, shape, walls, form):
+def _solver(lbm, Q, shape, walls, form, **kw):
     """form: D3Q27 the rate-1 relaxation, D3Q15 a force (a field)."""
     om = W.omegas(Q, 1 / 0.6) if Q == 27 and form else W.random_omegas(Q, seed=12)
     F = np.asarray(W.rng(13).uniform(-2e-3, 2e-3, (3,) + shape), dtype=np.float32)
     if Q == 15 and not form:
         F = np.zeros(3)
-    return lbm.Solver(Q, shape, om, walls=walls, force=F), om, F.astype(np.float64)
+    return lbm.Solver(Q, shape, om, walls=walls, force=F, **kw), om, F.astype(np.float64)
 
 
 @pytest.mark.parametrize("Q", [27, 15])
@@ -63,3 +63,23 @@ def test_results_do_not_depend_on_the_padding(lbm, Q, walls, shape):
         out.append(S.get_state())
     assert torch.isfinite(out[0]).all()
     assert torch.equal(*out)
+
+
+@pytest.mark.parametrize("Q", [27, 15])
+@pytest.mark.parametrize("storage", ["f16", "bf16"])
+@pytest.mark.parametrize("walls", [0, 3])
+@pytest.mark.parametrize("form", [False, True])
+@pytest.mark.parametrize("shape", [(3, 4, 9), (5, 6, 33)] + SHAPES)  # one- and two-cell
+def test_16bit_step_matches_oracle(lbm, Q, storage, walls, form, shape):
+    """One step from a state as stored against the FP64 oracle: what is stored is
+    (f - w) / w, below 2 here, rounded up or down."""
+    import oracle
+    w = oracle.equilibrium(Q, np.ones((1, 1, 1)), np.zeros((3, 1, 1, 1)), np.zeros(3))
+    S, om, F = _solver(lbm, Q, shape, walls, form, storage=storage)
+    S.set_state(w * (1 + W.rng(15).uniform(-0.2, 0.2, (Q,) + shape)))
+    f = S.get_state().cpu().numpy()
+    S.step(1)
+    want = oracle.run(Q, shape, f, F, om, 1, bc=walls)
+    assert np.abs(want / w - 1).max() < 1.5  # and BF16 references below 0.5
+    ulp = 2.0 ** (-10 if storage == "f16" else -7)
+    assert (np.abs(S.get_state().cpu().numpy() - want) <= w * ulp + 2e-6).all()
