@@ -59,6 +59,41 @@ struct AdjointArgs {
     float *gF;                  // dense [3][N] accumulator or nullptr
 };
 
+// The adjoint step, one cell per thread, for small grids with rows of odd length
+// (see step1_kernel); the adjoint is pulled from the mirrored neighbours x + e_q.
+template <int Q, typename T, bool kWalls, bool kEq>
+__global__ void __launch_bounds__(128) adjoint1_kernel(const StepIO<T> io, const AdjointArgs g,
+                                                       const StepArgs a) {
+    int x, y, z;
+    if (!cell_coords(a.g, x, y, z)) return;
+    const Rows<kWalls> R = pull_rows<kWalls>(a.g, y, z);
+    const int xs[3] = {(x + 1 == a.g.nx) ? 0 : x + 1, x, (x == 0) ? a.g.nx - 1 : x - 1};
+    float f[Q], mu[Q];
+    pull_cell<Q, T, false>(io, R, x, a.g.nx, f);
+    static_for<Q>([&](auto iq) {
+        constexpr int q = decltype(iq)::value;
+        constexpr int i = ex<Q>(q) + 1, j = ey<Q>(q) + 1, k = ez<Q>(q) + 1;
+        const bool wall = kWalls && R.wall[2 - j][2 - k];
+        const int src = wall ? R.own + x : R.off[2 - j][2 - k] + xs[2 - i];
+        mu[q] = Pair<float>::ld1(element<false>(g.lam_next[wall ? opposite<Q>(q) : q], src));
+    });
+    const long long N = (long long)a.g.nx * a.g.ny * a.g.nz;
+    const long long c = dense_index(a.g, x, y, z);
+    float Fx, Fy, Fz;
+    cell_force(a, c, N, Fx, Fy, Fz);
+    const typename Rates<Q>::type r = load_rates<Q>(a);
+    float lam[Q], gF[3];
+    adjoint_collide<kEq, float>(f, Fx, Fy, Fz, r, mu, lam, gF[0], gF[1], gF[2]);
+    static_for<Q>([&](auto iq) {
+        constexpr int q = decltype(iq)::value;
+        __stcs(element<false>(g.lam_out[q], R.own + x), lam[q]);
+    });
+    if (g.gF) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) g.gF[d * N + c] += gF[d];
+    }
+}
+
 // The pair's adjoints of its post-collision values, from the mirrored
 // neighbours; kSel: with the wall selects.
 template <int Q, bool kSel, bool kWalls, bool kRag>
@@ -237,6 +272,14 @@ __global__ void __launch_bounds__(128, 8) energy_kernel(const StepIO<T> io, cons
     }
 }
 
+// Grids of odd rows take the one-cell adjoint kernel up to this many warps on an SM
+// (kOneCellWarps).  us a step, one / two cells per thread, FP32, periodic / walled:
+// D3Q27 at general rates 21^3 (4 warps) 4.17 / 6.09, 29^3 (8) 5.18 / 6.61, 33^3 (16)
+// 6.59 / 6.47; walled 4.49 / 6.06, 5.34 / 6.44, 7.47 / 6.91; D3Q15 periodic 21^3 3.50 /
+// 3.91, 29^3 4.00 / 4.14, walled 3.65 / 3.86, 4.15 / 4.00.
+template <int Q>
+constexpr int kOneCellAdjointWarps = Q == 27 ? 8 : 4;
+
 template <int Q, typename T>
 cudaError_t launch_adjoint(const void *f_t, const float *lam_next, float *lam_out, float *gF,
                            const StepArgs &a, cudaStream_t st) {
@@ -247,11 +290,18 @@ cudaError_t launch_adjoint(const void *f_t, const float *lam_next, float *lam_ou
         g.lam_out[q] = lam_out + q * a.g.pop;
     }
     g.gF = gF;
+    const CellLaunch one = cell_launch(a.g);
+    const bool one_cell =
+        a.g.nx % 2 && a.g.nx > 1 && one.sm_warps() <= kOneCellAdjointWarps<Q>;
     const CellLaunch L = pair_launch(a.g, stored_row<float>(a.g.nx));
     const PackedRates pr = packed_rates(a);
     const auto launch = [&](auto eq) {
         constexpr bool kEq = decltype(eq)::value;
-        if (ragged<float>(a.g))  // one form, with the wall selects: the rarer case
+        if (one_cell && a.g.bc)
+            adjoint1_kernel<Q, T, true, kEq><<<one.grid, one.block, 0, st>>>(io, g, a);
+        else if (one_cell)
+            adjoint1_kernel<Q, T, false, kEq><<<one.grid, one.block, 0, st>>>(io, g, a);
+        else if (ragged<float>(a.g))  // one form, with the wall selects: the rarer case
             adjoint2_kernel<Q, T, true, true, kEq><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
         else if (a.g.bc)
             adjoint2_kernel<Q, T, true, false, kEq><<<L.grid, L.block, 0, st>>>(io, g, a, pr);

@@ -83,3 +83,30 @@ def test_16bit_step_matches_oracle(lbm, Q, storage, walls, form, shape):
     assert np.abs(want / w - 1).max() < 1.5  # and BF16 references below 0.5
     ulp = 2.0 ** (-10 if storage == "f16" else -7)
     assert (np.abs(S.get_state().cpu().numpy() - want) <= w * ulp + 2e-6).all()
+
+
+@pytest.mark.parametrize("Q", [27, 15])
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("walls", [0, 3])
+@pytest.mark.parametrize("general", [False, True])
+def test_adjoint_of_an_odd_row_equals_the_row_twice_over(lbm, Q, storage, walls, general):
+    """The state is at rest in the 16-bit types (their rounding depends on the pair)."""
+    shape = SHAPES[1]
+    om = W.omegas(Q, 1 / 0.6)
+    if general:
+        om[9:] = 1.1
+    f = W.random_field_state(shape, Q, spread=0.2 if storage == "f32" else 0.0)
+    F = W.rng(16).uniform(-1e-2, 1e-2, (3,) + shape)
+    lam = W.rng(17).standard_normal((Q,) + shape)
+    got = []
+    for k in (1, 2):
+        S = lbm.Solver(Q, shape[:2] + (k * shape[2],), om, walls=walls, storage=storage,
+                       force=np.concatenate([F] * k, -1))
+        S.set_state(np.concatenate([f] * k, -1))
+        a, b = S.new_adjoint_field(), S.new_adjoint_field()
+        S.adjoint_view(a).copy_(torch.as_tensor(np.concatenate([lam] * k, -1)))
+        gF = torch.zeros((3,) + S.shape, dtype=torch.float32, device="cuda")
+        S.adjoint_step(S.current_buffer(), a, b, gF)
+        got.append([v[..., :shape[2]].double().cpu().numpy() for v in (S.adjoint_view(b), gF)])
+    for one, two in zip(*got):  # 1000 FP32 operations on O(1) values
+        np.testing.assert_allclose(one, two, rtol=0, atol=1e-5 * np.abs(two).max())
