@@ -1435,7 +1435,19 @@ void launch_step_kernel(const StepIO<T> &io, const StepArgs &a, const PackedRate
     // grids of short rows are small, and a second copy of the loads (pull_pairs)
     // costs them more than it saves: D3Q27 FP32 between walls, 16^3 3.55 / 3.05
     // us, 16 x 64 x 64 4.13 / 3.75 us with / without it
-    const bool is_short = L.block.x < 32 && !ragged<T>(a.g);
+    const bool is_short = L.block.x < 32 && (Storage<T>::kRef || !ragged<T>(a.g));
+    if constexpr (Storage<T>::kRef && kWalls) {
+        // BF16 in ragged rows too (24^3: D3Q27 5.1 / 5.7, D3Q15 2.76 / 2.89; FP32 and FP16
+        // up to 7 % slower)
+        if (is_short && ragged<T>(a.g)) {
+            if constexpr (Q == 27)
+                step2_kernel<T, true, kForm, true, true><<<L.grid, L.block, 0, st>>>(io, a, pr);
+            else
+                step2_q15_kernel<T, true, kForm, true, true>
+                    <<<L.grid, L.block, 0, st>>>(io, a, pr);
+            return;
+        }
+    }
     if constexpr (Q == 27) {
         if constexpr (kWalls) {
             if (is_short) {
