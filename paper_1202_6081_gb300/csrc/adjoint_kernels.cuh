@@ -120,7 +120,7 @@ __device__ __forceinline__ void pull_adjoint(const AdjointArgs &g, const Rows<kW
 // 206 us).  The rate-1 form (kEq, adjoint27) needs fewer and takes 4 blocks, 128
 // registers: 128^3 in 113.8 us, 6.64 TB/s, where the general form took 135; FP16
 // states 114 / 119 us at 4 / 3 blocks; 3 blocks for BF16 states (117 / 126 at 4)
-// and ragged rows (126 x 128 x 128 walled 121 / 130).
+// and ragged rows (126 x 128 x 128 walled 122 / 127).
 // kRag: ragged rows (PairCols).
 template <typename T, bool kRag, bool kEq>
 constexpr int kAdjointBlocks = kEq && !kRag && !Storage<T>::kRef ? 4 : 3;
@@ -295,14 +295,20 @@ cudaError_t launch_adjoint(const void *f_t, const float *lam_next, float *lam_ou
         a.g.nx % 2 && a.g.nx > 1 && one.sm_warps() <= kOneCellAdjointWarps<Q>;
     const CellLaunch L = pair_launch(a.g, stored_row<float>(a.g.nx));
     const PackedRates pr = packed_rates(a);
+    // ragged periodic rows without the wall selects (us a step, FP32, with / without:
+    // D3Q27 30^3 5.8 / 3.8, at general rates 6.5 / 4.8, 126 x 128 x 128 120 / 117; D3Q15
+    // 30^3 4.0 / 3.4), but not D3Q15 in longer rows (126 x 128 x 128 82.6 / 100)
+    const bool periodic_form = Q == 27 || L.block.x < 32;
     const auto launch = [&](auto eq) {
         constexpr bool kEq = decltype(eq)::value;
         if (one_cell && a.g.bc)
             adjoint1_kernel<Q, T, true, kEq><<<one.grid, one.block, 0, st>>>(io, g, a);
         else if (one_cell)
             adjoint1_kernel<Q, T, false, kEq><<<one.grid, one.block, 0, st>>>(io, g, a);
-        else if (ragged<float>(a.g))  // one form, with the wall selects: the rarer case
+        else if (ragged<float>(a.g) && (a.g.bc || !periodic_form))
             adjoint2_kernel<Q, T, true, true, kEq><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
+        else if (ragged<float>(a.g))
+            adjoint2_kernel<Q, T, false, true, kEq><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
         else if (a.g.bc)
             adjoint2_kernel<Q, T, true, false, kEq><<<L.grid, L.block, 0, st>>>(io, g, a, pr);
         else
