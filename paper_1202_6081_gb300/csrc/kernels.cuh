@@ -352,8 +352,9 @@ __device__ __forceinline__ Rows<kWalls> pull_rows(const Grid &g, int y, int z) {
 // Cells a row's stores cover: the row rounded up to whole 32-byte sectors (the
 // pitch has room).  A sector that is stored in part has to be filled from DRAM:
 // D3Q27 FP32 at 126 x 117 x 133 cells took 76.2 us a step, at 128 (no partial
-// sector) 64.9 us.  The threads past the row's end repeat its last cells and
-// store them there, in the same instructions as the rest of their warp.
+// sector) 64.9 us.  The threads past the row's end store there in the same
+// instructions as the rest of their warp: the row's last cells again, in place what
+// they make of the padding itself (PairCols), the adjoint step zeros (zero_padding).
 template <typename T>
 __host__ __device__ constexpr int stored_row(int nx) {
     constexpr int n = 32 / int(sizeof(T));
@@ -1026,8 +1027,9 @@ __device__ __forceinline__ float4 pair_collide(const StepIO<T> &io, const StepAr
 // Element offsets instead of byte offsets (element()) where those measured slower
 // in the in-place kernels: 256^3 us a step, bytes / elements, D3Q27 BF16 466 / 411
 // (452 with row and column summed first), FP32 at general rates 545 / 527 (598);
-// ragged rows (250 x 256 x 256, a wall) FP16 511 / 356 (407 row first); else
-// bytes: D3Q27 FP16 321 / 353, D3Q15 FP16 203 / 231.
+// ragged rows (250 x 256 x 256) D3Q27 FP16 between walls 348 / 339 (340), though
+// periodic 319 / 329 and D3Q15 FP16 200 / 214; else bytes: D3Q27 FP16 320 / 353,
+// D3Q15 FP16 204 / 231.
 template <int Q, typename T, bool kEq, bool kRag>
 constexpr bool kAAPlain = kRag || (Q == 27 && (Storage<T>::kRef || (sizeof(T) == 4 && !kEq)));
 
